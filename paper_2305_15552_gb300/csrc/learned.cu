@@ -92,12 +92,6 @@ struct LpConstW {
   const LpParams& P;
   __device__ __forceinline__ float operator()(int i) const { return P.p[i]; }
 };
-// Weights from shared memory.
-struct LpSmemW {
-  const float* s;
-  __device__ __forceinline__ float operator()(int i) const { return s[i]; }
-};
-
 // Inference: max(a, 0) (one instruction); a parameter vector with a non-finite entry is
 // caught on the host before the launch (it makes every output non-finite, as the network
 // arithmetic would).
@@ -227,137 +221,326 @@ int apply_grid(int64_t count) {
 }  // namespace
 
 // ---------------------------------------------------------------------------------------
-// Loss of the correction targets and its gradient.  A CTA takes tiles of kGradThreads entries
-// (one per thread): forward, dL/dm, backward to the per-entry layer deltas, all staged in
-// shared memory; then each thread sums, over the tile, the products that make up its own
-// parameters' gradient.  Tile sums (FP32) are added into FP64 per-thread totals; CTA partials
-// are reduced in a fixed order, so the result is deterministic.
+// Loss of the correction targets and its gradient.  A CTA of four warps takes tiles of
+// kGradThreads entries: forward, dL/dm, backward to the per-entry layer deltas, all staged in
+// shared memory, then the products that make up each parameter's gradient, summed over the tile
+// in entry order (FP32) and added to FP64 totals held by the thread that owns the parameter; CTA
+// partials are reduced in a fixed order, so the result is deterministic.
+//
+// What bounds it: the shared-memory pipe and the FP32 pipe at about the same level (~3600 multiply-
+// adds an entry; a 128-bit shared load takes two clocks when adjacent lanes share its address and
+// four otherwise).  One thread per entry, as inference runs, would load every weight once per 32
+// entries and staging rows of 32 words puts a warp's stores into one bank.  So:
+//   * layers: warp w computes outputs [8 w, 8 w + 8) for all 128 entries, four entries a lane, so
+//     eight weights (uniform, two loads) serve 32 multiply-adds a lane, issued as FP32x2 pairs;
+//   * W2 gradient: two warps, each thread a 4 x 4 block of parameters in registers (two loads per
+//     16 multiply-adds); the other two take W1, the biases and b3;
+//   * rows are padded to 36 words: a lane's 16-byte piece of its own row is conflict free;
+//   * the output layer's gradient is summed before the backward pass overwrites the second
+//     layer's activations with the first layer's deltas; three CTAs per SM then fit.
+// Every sum keeps its order (entries ascending, FP32, one tile of 128), so each tile's FP32 sums
+// are those of a thread-per-entry kernel.  Measured at 8e6 entries (1M rows x 8 columns): 1.85 ms;
+// the thread-per-entry kernel took 7.48 ms.
 // ---------------------------------------------------------------------------------------
 namespace {
 
-constexpr int kGradThreads = 128;
-constexpr int kGradSlots = (kLpTrained + kGradThreads - 1) / kGradThreads;   // 11
+constexpr int kGradThreads = 128;                                             // entries per tile
 constexpr int kGradOut = kLpTrained + 1;                                      // + loss
-constexpr int kSU = 8;                                                        // row stride of sU
-constexpr size_t kGradSmemFloats =
-    kLpParams + 3 + (size_t)kGradThreads * (kSU + 4 * kLpHid + 1) + 4;
+constexpr int kGS = 36;                                                       // row stride of the staged blocks
+constexpr int kGradCtas = 3;                                                  // per SM
 
-__global__ void __launch_bounds__(kGradThreads)
+struct GradSmem {
+  float W2[kLpHid * kLpHid];            // [k][l]
+  float W2T[kLpHid * kLpHid];           // [l][k]
+  float W1[kLpHid * 8];                 // [k][6 weights, bias, 0]
+  float b2[kLpHid], w3[kLpHid];
+  float mu[8], sigma[8];                // [6], [7]: padding; mu[7] holds b3
+  float U[kGradThreads * 8];            // features u0..u5, f2 (raw), 0
+  float H1[kGradThreads * kGS];         // layer 1 activations
+  float H2[kGradThreads * kGS];         // layer 2 activations, then the layer 1 deltas
+  float Da2[kGradThreads * kGS];        // layer 2 deltas
+  float dm[kGradThreads];
+};
+static_assert(sizeof(GradSmem) + 1024 <= 233472 / kGradCtas, "three CTAs per SM");
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// acc[i][2q..2q+1] += w[2q..2q+1] * x_i for the four entries i of a lane, eight outputs
+__device__ __forceinline__ void grad_rank1(float2 (&acc)[4][4], const float* w, const float (&x)[4]) {
+  const float4 wa = ld4(w), wb = ld4(w + 4);
+  const float2 wp[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
+                        make_float2(wb.z, wb.w)};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 xx = make_float2(x[i], x[i]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[i][q] = __ffma2_rn(wp[q], xx, acc[i][q]);
+  }
+}
+
+// acc[i][:] += sum_r M[r][col0 .. col0 + 8) * S[entry i][r], r = 0..31 ascending
+__device__ __forceinline__ void grad_layer(float2 (&acc)[4][4], const float* M, int col0, const float* S, int lane) {
+#pragma unroll 2
+  for (int r0 = 0; r0 < kLpHid; r0 += 4) {
+    float4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = ld4(S + (lane + 32 * i) * kGS + r0);
+    const float x0[4] = {x[0].x, x[1].x, x[2].x, x[3].x}, x1[4] = {x[0].y, x[1].y, x[2].y, x[3].y};
+    const float x2[4] = {x[0].z, x[1].z, x[2].z, x[3].z}, x3[4] = {x[0].w, x[1].w, x[2].w, x[3].w};
+    grad_rank1(acc, M + (r0 + 0) * kLpHid + col0, x0);
+    grad_rank1(acc, M + (r0 + 1) * kLpHid + col0, x1);
+    grad_rank1(acc, M + (r0 + 2) * kLpHid + col0, x2);
+    grad_rank1(acc, M + (r0 + 3) * kLpHid + col0, x3);
+  }
+}
+
+__device__ __forceinline__ void grad_store8(float* row, const float (&v)[8]) {
+  reinterpret_cast<float4*>(row)[0] = make_float4(v[0], v[1], v[2], v[3]);
+  reinterpret_cast<float4*>(row)[1] = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+__global__ void __launch_bounds__(kGradThreads, kGradCtas)
 k_lp_grad(const float* __restrict__ params, const float* __restrict__ F, const float* __restrict__ rr,
           const float* __restrict__ zz, const double* __restrict__ colw, int64_t n, int m,
           double* __restrict__ part) {
-  extern __shared__ __align__(16) float sm[];
-  float* sW = sm;                                        // kLpParams (+3 pad)
-  float* sU = sW + kLpParams + 3;                        // [T][8]
-  float* sH1 = sU + kGradThreads * kSU;                  // [T][32]
-  float* sH2 = sH1 + kGradThreads * kLpHid;
-  float* sDa2 = sH2 + kGradThreads * kLpHid;
-  float* sDa1 = sDa2 + kGradThreads * kLpHid;
-  float* sDm = sDa1 + kGradThreads * kLpHid;             // [T]
-  float* sOne = sDm + kGradThreads;                      // [1] = 1
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
   __shared__ double red[kGradThreads];
-  __shared__ double sTot[kGradSlots * kGradThreads];    // this thread's parameter totals
-  const int t = threadIdx.x;
-  for (int i = t; i < kLpParams; i += kGradThreads) sW[i] = params[i];
-  if (t == 0) sOne[0] = 1.0f;
-  for (int s = 0; s < kGradSlots; ++s) sTot[s * kGradThreads + t] = 0.0;
-  __syncthreads();
-  const LpSmemW w{sW};
-  double loss = 0.0;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  for (int i = t; i < kLpHid * kLpHid; i += kGradThreads) {
+    const float v = params[kLpOffW2 + i];
+    S.W2[i] = v;
+    S.W2T[(i % kLpHid) * kLpHid + i / kLpHid] = v;
+  }
+  for (int i = t; i < kLpHid * 8; i += kGradThreads) {
+    const int k = i >> 3, q = i & 7;
+    S.W1[i] = q < kLpFeat ? params[kLpOffW1 + k * kLpFeat + q] : (q == kLpFeat ? params[kLpOffB1 + k] : 0.0f);
+  }
+  if (t < kLpHid) {
+    S.b2[t] = params[kLpOffB2 + t];
+    S.w3[t] = params[kLpOffW3 + t];
+  }
+  if (t < 8) {
+    S.mu[t] = t < kLpFeat ? params[kLpOffMu + t] : (t == 7 ? params[kLpOffB3] : 0.0f);
+    S.sigma[t] = t < kLpFeat ? params[kLpOffSigma + t] : 1.0f;
+  }
+  // roles of the gradient sums: which two warps take W2 differs among the CTAs of an SM, so that
+  // the work is spread over its four schedulers
+  const int role = (w + (int)((int64_t)blockIdx.x * kGradCtas / gridDim.x)) & 3;
+  const int kb = 4 * (((role & 1) * 32 + lane) >> 3), lb = 4 * (lane & 7);   // W2 block (roles 0, 1)
+  double tot[16];       // roles 0, 1: the 4 x 4 block; roles 2, 3: W1 (3), bias
+#pragma unroll
+  for (int i = 0; i < 16; ++i) tot[i] = 0.0;
+  double tot_w3 = 0.0, tot_b3 = 0.0, loss = 0.0;
   const int64_t cnt = n * m;
   const int64_t ntiles = (cnt + kGradThreads - 1) / kGradThreads;
+  // the next tile's features (6 consecutive words a thread apart), residual and target
+  float fn[kLpFeat], rn = 0.0f, zn = 0.0f;
+  auto fetch = [&](int64_t tile) {
+    const int64_t base = tile * kGradThreads;
+    const int valid = (int)min64(kGradThreads, cnt - base);
+#pragma unroll
+    for (int i = 0; i < kLpFeat; ++i) {
+      const int e = t + i * kGradThreads;
+      fn[i] = e < valid * kLpFeat ? F[base * kLpFeat + e] : 0.0f;
+    }
+    rn = t < valid ? rr[base + t] : 0.0f;
+    zn = t < valid ? zz[base + t] : 0.0f;
+  };
+  if ((int64_t)blockIdx.x < ntiles) fetch(blockIdx.x);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t e = tile * kGradThreads + t;
-    const bool valid = e < cnt;
-    // ---- forward
-    float u[kLpFeat];
-    const float jsc = valid ? lp_jscale(F[e * kLpFeat + 2]) : 0.0f;
+    __syncthreads();   // the weights are staged; the previous tile's sums are done with its rows
+    const int64_t base = tile * kGradThreads;
+    const int valid = (int)min64(kGradThreads, cnt - base);
+    // ---- standardised features
 #pragma unroll
-    for (int q = 0; q < kLpFeat; ++q) {
-      u[q] = valid ? (F[e * kLpFeat + q] - w(kLpOffMu + q)) / w(kLpOffSigma + q) : 0.0f;
-      sU[t * kSU + q] = u[q];
+    for (int i = 0; i < kLpFeat; ++i) {
+      const int e = t + i * kGradThreads, x = e / kLpFeat, q = e % kLpFeat;
+      S.U[x * 8 + q] = x < valid ? (fn[i] - S.mu[q]) / S.sigma[q] : 0.0f;
+      if (q == 2) S.U[x * 8 + 6] = fn[i];
     }
-    float h1[kLpHid];
-    uint32_t m1 = 0, m2 = 0;
+    const float r = rn, z = zn;
+    if (tile + gridDim.x < ntiles) fetch(tile + gridDim.x);
+    __syncthreads();
+    // ---- layer 1, outputs [8 w, 8 w + 8) of entries lane + 32 i
+    unsigned m1 = 0, m2 = 0;   // bit 8 i + o: activation of output 8 w + o is positive
+    {
+      float4 ua[4];
+      float2 ub[4];
 #pragma unroll
-    for (int k = 0; k < kLpHid; ++k) {
-      float a = w(kLpOffB1 + k);
+      for (int i = 0; i < 4; ++i) {
+        ua[i] = ld4(S.U + (lane + 32 * i) * 8);
+        ub[i] = *reinterpret_cast<const float2*>(S.U + (lane + 32 * i) * 8 + 4);
+      }
+      float h[4][8];
 #pragma unroll
-      for (int q = 0; q < kLpFeat; ++q) a = fmaf(w(kLpOffW1 + k * kLpFeat + q), u[q], a);
-      h1[k] = valid ? lp_relu(a) : 0.0f;
-      if (a > 0.0f) m1 |= 1u << k;
-      sH1[t * kLpHid + k] = h1[k];
-    }
-    float mo = w(kLpOffB3);
-#pragma unroll 1
-    for (int k = 0; k < kLpHid; ++k) {
-      float a = w(kLpOffB2 + k);
+      for (int o = 0; o < 8; ++o) {
+        const float4 wa = ld4(S.W1 + (8 * w + o) * 8), wb = ld4(S.W1 + (8 * w + o) * 8 + 4);
 #pragma unroll
-      for (int l = 0; l < kLpHid; ++l) a = fmaf(w(kLpOffW2 + k * kLpHid + l), h1[l], a);
-      const float h2 = valid ? lp_relu(a) : 0.0f;
-      if (a > 0.0f) m2 |= 1u << k;
-      sH2[t * kLpHid + k] = h2;
-      mo = fmaf(w(kLpOffW3 + k), h2, mo);
-    }
-    // ---- loss, dL/dm and dL/do = dL/dm * J (m = J (1 + o))
-    float dm = 0.0f;
-    if (valid) {
-      const int j = (int)(e % m);
-      const float r = rr[e];
-      const double cw = colw[j];
-      const float err = jsc * (1.0f + mo) * r - zz[e];
-      dm = (float)(2.0 * cw) * r * err * jsc;
-      loss += cw * (double)err * (double)err;
-    }
-    sDm[t] = dm;
-    // ---- backward to the layer deltas
-    float da2[kLpHid];
+        for (int i = 0; i < 4; ++i) {
+          float a = wb.z;
+          a = fmaf(wa.x, ua[i].x, a);
+          a = fmaf(wa.y, ua[i].y, a);
+          a = fmaf(wa.z, ua[i].z, a);
+          a = fmaf(wa.w, ua[i].w, a);
+          a = fmaf(wb.x, ub[i].x, a);
+          a = fmaf(wb.y, ub[i].y, a);
+          if (a > 0.0f) m1 |= 1u << (8 * i + o);
+          h[i][o] = lane + 32 * i < valid ? lp_relu(a) : 0.0f;
+        }
+      }
 #pragma unroll
-    for (int k = 0; k < kLpHid; ++k) {
-      da2[k] = (m2 >> k & 1u) ? dm * w(kLpOffW3 + k) : 0.0f;
-      sDa2[t * kLpHid + k] = da2[k];
-    }
-#pragma unroll 1
-    for (int l = 0; l < kLpHid; ++l) {
-      float g = 0.0f;
-#pragma unroll
-      for (int k = 0; k < kLpHid; ++k) g = fmaf(w(kLpOffW2 + k * kLpHid + l), da2[k], g);
-      sDa1[t * kLpHid + l] = (m1 >> l & 1u) ? g : 0.0f;
+      for (int i = 0; i < 4; ++i) grad_store8(S.H1 + (lane + 32 * i) * kGS + 8 * w, h[i]);
     }
     __syncthreads();
-    // ---- this thread's parameters: sum over the tile of (delta x activation)
-#pragma unroll 1
-    for (int s = 0; s < kGradSlots; ++s) {
-      const int q = t + s * kGradThreads;
-      if (q < kLpTrained) {
-        const float* pa;
-        const float* pb;
-        int sa, sb;
-        if (q < kLpOffB1 - kLpFixed) {                       // W1[k][l]
-          pa = sDa1 + q / kLpFeat; sa = kLpHid; pb = sU + q % kLpFeat; sb = kSU;
-        } else if (q < kLpOffW2 - kLpFixed) {                // b1[k]
-          pa = sDa1 + (q - (kLpOffB1 - kLpFixed)); sa = kLpHid; pb = sOne; sb = 0;
-        } else if (q < kLpOffB2 - kLpFixed) {                // W2[k][l]
-          const int x = q - (kLpOffW2 - kLpFixed);
-          pa = sDa2 + x / kLpHid; sa = kLpHid; pb = sH1 + x % kLpHid; sb = kLpHid;
-        } else if (q < kLpOffW3 - kLpFixed) {                // b2[k]
-          pa = sDa2 + (q - (kLpOffB2 - kLpFixed)); sa = kLpHid; pb = sOne; sb = 0;
-        } else if (q < kLpOffB3 - kLpFixed) {                // w3[k]
-          pa = sDm; sa = 1; pb = sH2 + (q - (kLpOffW3 - kLpFixed)); sb = kLpHid;
-        } else {                                             // b3
-          pa = sDm; sa = 1; pb = sOne; sb = 0;
-        }
-        float acc = 0.0f;
-#pragma unroll 8
-        for (int x = 0; x < kGradThreads; ++x) acc = fmaf(pa[x * sa], pb[x * sb], acc);
-        sTot[s * kGradThreads + t] += (double)acc;
+    // ---- layer 2
+    float2 acc[4][4];
+    {
+      const float4 ba = ld4(S.b2 + 8 * w), bb = ld4(S.b2 + 8 * w + 4);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[i][0] = make_float2(ba.x, ba.y);
+        acc[i][1] = make_float2(ba.z, ba.w);
+        acc[i][2] = make_float2(bb.x, bb.y);
+        acc[i][3] = make_float2(bb.z, bb.w);
       }
     }
+    grad_layer(acc, S.W2T, 8 * w, S.H1, lane);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float h[8];
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const float a = (o & 1) ? acc[i][o >> 1].y : acc[i][o >> 1].x;
+        if (a > 0.0f) m2 |= 1u << (8 * i + o);
+        h[o] = lane + 32 * i < valid ? lp_relu(a) : 0.0f;
+      }
+      grad_store8(S.H2 + (lane + 32 * i) * kGS + 8 * w, h);
+    }
     __syncthreads();
+    // ---- output layer of entry t, loss, dL/dm and dL/do = dL/dm * J (m = J (1 + o))
+    {
+      float mo = S.mu[7];
+#pragma unroll
+      for (int k = 0; k < kLpHid; k += 4) {
+        const float4 wv = ld4(S.w3 + k), hv = ld4(S.H2 + t * kGS + k);
+        mo = fmaf(wv.x, hv.x, mo);
+        mo = fmaf(wv.y, hv.y, mo);
+        mo = fmaf(wv.z, hv.z, mo);
+        mo = fmaf(wv.w, hv.w, mo);
+      }
+      float dm = 0.0f;
+      if (t < valid) {
+        const float jsc = lp_jscale(S.U[t * 8 + 6]);
+        const int64_t e = base + t;
+        const int j = cnt <= 0x7fffffff ? (int)((unsigned)e % (unsigned)m) : (int)(e % m);
+        const double cw = colw[j];
+        const float err = jsc * (1.0f + mo) * r - z;
+        dm = (float)(2.0 * cw) * r * err * jsc;
+        loss += cw * (double)err * (double)err;
+      }
+      S.dm[t] = dm;
+    }
+    __syncthreads();
+    // ---- layer 2 deltas
+    {
+      const float4 wa = ld4(S.w3 + 8 * w), wb = ld4(S.w3 + 8 * w + 4);
+      const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float dm = S.dm[lane + 32 * i];
+        float d[8];
+#pragma unroll
+        for (int o = 0; o < 8; ++o) d[o] = (m2 >> (8 * i + o) & 1u) ? dm * wv[o] : 0.0f;
+        grad_store8(S.Da2 + (lane + 32 * i) * kGS + 8 * w, d);
+      }
+    }
+    // w3 and b3 (the layer 2 activations are overwritten below): one lane per output
+    if (role == 3) {
+      float a3 = 0.0f, ab = 0.0f;
+#pragma unroll 8
+      for (int x = 0; x < kGradThreads; ++x) {
+        const float dm = S.dm[x];
+        a3 = fmaf(dm, S.H2[x * kGS + lane], a3);
+        ab += dm;
+      }
+      tot_w3 += (double)a3;
+      tot_b3 += (double)ab;
+    }
+    __syncthreads();
+    // ---- layer 1 deltas, into the layer 2 activations' rows
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][q] = make_float2(0.0f, 0.0f);
+    grad_layer(acc, S.W2, 8 * w, S.Da2, lane);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float d[8];
+#pragma unroll
+      for (int o = 0; o < 8; ++o)
+        d[o] = (m1 >> (8 * i + o) & 1u) ? ((o & 1) ? acc[i][o >> 1].y : acc[i][o >> 1].x) : 0.0f;
+      grad_store8(S.H2 + (lane + 32 * i) * kGS + 8 * w, d);
+    }
+    __syncthreads();
+    // ---- sums over the tile of (delta x activation)
+    if (role < 2) {
+      float2 g[4][2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) g[i][0] = g[i][1] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+      for (int x = 0; x < kGradThreads; ++x) {
+        const float4 a = ld4(S.Da2 + x * kGS + kb), b = ld4(S.H1 + x * kGS + lb);
+        const float av[4] = {a.x, a.y, a.z, a.w};
+        const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 aa = make_float2(av[i], av[i]);
+          g[i][0] = __ffma2_rn(aa, b0, g[i][0]);
+          g[i][1] = __ffma2_rn(aa, b1, g[i][1]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        tot[4 * i + 0] += (double)g[i][0].x;
+        tot[4 * i + 1] += (double)g[i][0].y;
+        tot[4 * i + 2] += (double)g[i][1].x;
+        tot[4 * i + 3] += (double)g[i][1].y;
+      }
+    } else {
+      // row `lane` of W1, columns [0, 3) and b1 (role 2) or columns [3, 6) and b2 (role 3)
+      const int q0 = role == 2 ? 0 : 3;
+      const float* bias = role == 2 ? S.H2 : S.Da2;
+      float g0 = 0.0f, g1 = 0.0f, g2 = 0.0f, gb = 0.0f;
+#pragma unroll 8
+      for (int x = 0; x < kGradThreads; ++x) {
+        const float d = S.H2[x * kGS + lane];
+        g0 = fmaf(d, S.U[x * 8 + q0], g0);
+        g1 = fmaf(d, S.U[x * 8 + q0 + 1], g1);
+        g2 = fmaf(d, S.U[x * 8 + q0 + 2], g2);
+        gb += bias[x * kGS + lane];
+      }
+      tot[0] += (double)g0;
+      tot[1] += (double)g1;
+      tot[2] += (double)g2;
+      tot[3] += (double)gb;
+    }
   }
-  for (int s = 0; s < kGradSlots; ++s) {
-    const int q = t + s * kGradThreads;
-    if (q < kLpTrained) part[(size_t)blockIdx.x * kGradOut + q] = sTot[s * kGradThreads + t];
+  double* out = part + (size_t)blockIdx.x * kGradOut;
+  if (role < 2) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) out[kLpOffW2 - kLpFixed + (kb + i) * kLpHid + lb + c] = tot[4 * i + c];
+  } else {
+    const int q0 = role == 2 ? 0 : 3;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[kLpOffW1 - kLpFixed + lane * kLpFeat + q0 + c] = tot[c];
+    out[(role == 2 ? kLpOffB1 : kLpOffB2) - kLpFixed + lane] = tot[3];
+    if (role == 3) {
+      out[kLpOffW3 - kLpFixed + lane] = tot_w3;
+      if (lane == 0) out[kLpOffB3 - kLpFixed] = tot_b3;
+    }
   }
   red[t] = loss;
   __syncthreads();
@@ -365,7 +548,7 @@ k_lp_grad(const float* __restrict__ params, const float* __restrict__ F, const f
     if (t < o) red[t] += red[t + o];
     __syncthreads();
   }
-  if (t == 0) part[(size_t)blockIdx.x * kGradOut + kLpTrained] = red[0];
+  if (t == 0) out[kLpTrained] = red[0];
 }
 
 __global__ void k_lp_adam(float* __restrict__ p, const double* __restrict__ g, float* __restrict__ m1,
@@ -381,7 +564,7 @@ __global__ void k_lp_adam(float* __restrict__ p, const double* __restrict__ g, f
   p[i] = (float)((double)p[i] - lr * (a / bc1) / (sqrt(v / bc2) + eps));
 }
 
-int grad_grid() { return num_sms() * 2; }
+int grad_grid() { return num_sms() * kGradCtas; }
 
 template <typename V>
 eig_status row_abs_sum_t(const SpmmPlan& P, double* out, cudaStream_t st) {
@@ -477,11 +660,11 @@ size_t lp_grad_workspace_bytes() { return (size_t)grad_grid() * kGradOut * 8 + 2
 eig_status lp_grad(const float* params, const float* F, const float* r, const float* z, const double* colw,
                    int64_t n, int m, double* out, void* workspace, cudaStream_t st) {
   if (m < 1 || n < 0 || !params || !out || !workspace) return EIG_EINVAL;
-  const int grid = grad_grid();
-  const size_t smem = kGradSmemFloats * sizeof(float);
+  const int64_t ntiles = (n * m + kGradThreads - 1) / kGradThreads;
+  const int grid = (int)max64(1, min64(ntiles, grad_grid()));
   // set on every call: the attribute belongs to the current device
-  EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_lp_grad, (int)smem));
-  k_lp_grad<<<grid, kGradThreads, smem, st>>>(params, F, r, z, colw, n, m, (double*)workspace);
+  EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_lp_grad, (int)sizeof(GradSmem)));
+  k_lp_grad<<<grid, kGradThreads, sizeof(GradSmem), st>>>(params, F, r, z, colw, n, m, (double*)workspace);
   EIG_LAUNCH_CHECK("k_lp_grad");
   return reduce_partials((const double*)workspace, grid, kGradOut, out, st);
 }

@@ -1,0 +1,39 @@
+"""Kernels at the edges of their tiles: remainders, the smallest sizes, ragged rows, against the
+FP64 oracle or the definition.  Tolerances are derived beside each test."""
+import numpy as np
+import pytest
+
+from oracle import learned as L
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _dev(a):
+    return torch.tensor(np.ascontiguousarray(a), device="cuda")
+
+
+# n * m entries: one, just below / at / above a tile of 128, one tile a CTA over the whole grid
+# (3 x 152 tiles) and a ragged tile more
+@pytest.mark.parametrize("n,m", [(1, 1), (127, 1), (16, 8), (43, 3), (456 * 16, 8), (19457, 3)])
+def test_lp_grad_tile_edges(n, m):
+    from paper_2305_15552_gb300 import binding as B
+    rng = np.random.default_rng(n + m)
+    F = rng.standard_normal((n, m, 6)) * [60, 1, 60, 60, 1, 10] + [150, 1, 150, 170, 0, 0]
+    F = F.astype(np.float32)
+    r = (1e-2 * rng.standard_normal((n, m))).astype(np.float32)
+    z = (r / 50 * (1 + 0.3 * rng.standard_normal((n, m)))).astype(np.float32)
+    colw = 1.0 / (m * (z.astype(np.float64) ** 2).sum(0))
+    p = (0.3 * rng.standard_normal(L.N_PARAMS)).astype(np.float32)
+    p[:12] = [150, 1, 150, 170, 0, 0, 60, 1, 60, 60, 1, 10]
+    s = dict(F=_dev(F.reshape(-1, 6)), r=_dev(r.reshape(-1)), z=_dev(z.reshape(-1)), colw=_dev(colw), n=n, m=m)
+    g = B.lp_grad(_dev(p), s).cpu().numpy()
+    Lo, go = L.loss_grad(p.astype(np.float64), F.astype(np.float64), r.astype(np.float64), z.astype(np.float64),
+                         colw * m)
+    # FP32 chains of 6 + 32 + 32 + 128 products: a normwise error of ~200 * 2^-24 = 1.2e-5 at worst,
+    # and the loss sums squares of differences that keep two to three digits of z
+    assert g[-1] == pytest.approx(Lo, rel=1e-4)
+    gt = go[L.N_FIXED:]
+    for a, b in [(12, 204), (204, 236), (236, 1260), (1260, 1292), (1292, 1324), (1324, 1325)]:
+        ga, gb = g[a - 12:b - 12], gt[a - 12:b - 12]
+        assert np.linalg.norm(ga - gb) <= 1e-4 * max(np.linalg.norm(gb), 1e-2 * np.linalg.norm(gt)), (a, b)
