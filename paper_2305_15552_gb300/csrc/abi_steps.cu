@@ -89,10 +89,10 @@ eig_status eig_gram(const void* A, const void* B, int64_t n, int nb, eig_dtype v
   AsyncScratch sc(st);
   EIG_TRY(sc.get(gram_scratch_bytes(1, nb)));
   BlockList bl;
-  bl.n = 2;
+  bl.n = A == B ? 1 : 2;
   bl.p[0] = A;
   bl.p[1] = B;
-  const int pa = 0, pb = 1;
+  const int pa = 0, pb = bl.n - 1;
   return gram_multi(bl, &pa, &pb, 1, nb, n, vec_type, G, sc.p, st);
 }
 

@@ -8,32 +8,8 @@
 namespace eig {
 
 // ---------------------------------------------------------------------------------------
-// double-float accumulation in FP32 (Knuth TwoSum + Fast2Sum)
+// Gram products
 // ---------------------------------------------------------------------------------------
-struct DF {
-  float hi, lo;
-};
-__device__ __forceinline__ void df_add(DF& a, float x) {
-  const float s = a.hi + x;
-  const float bb = s - a.hi;
-  const float err = (a.hi - (s - bb)) + (x - bb);
-  const float e = err + a.lo;
-  const float h = s + e;
-  a.lo = e - (h - s);
-  a.hi = h;
-}
-
-template <typename T> struct Acc;  // chunk accumulator type per vector type
-template <> struct Acc<float> { typedef DF type; };
-template <> struct Acc<double> { typedef double type; };
-
-__device__ __forceinline__ void acc_zero(DF& a) { a.hi = 0.f; a.lo = 0.f; }
-__device__ __forceinline__ void acc_zero(double& a) { a = 0.0; }
-__device__ __forceinline__ void acc_add(DF& a, float x) { df_add(a, x); }
-__device__ __forceinline__ void acc_add(double& a, double x) { a += x; }
-__device__ __forceinline__ double acc_get(const DF& a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ double acc_get(const double& a) { return a; }
-
 constexpr int kGramThreads = 256;
 constexpr int kGramRows = 32;
 
@@ -42,107 +18,154 @@ struct PairList {
   int n;
 };
 
-// 16-byte asynchronous global -> shared copy; src_bytes = 0 fills the 16 bytes with zeros.
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int src_bytes) {
+// 16-byte asynchronous global -> shared copy.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// One row of a thread's TM x TM tile: its TM values of each block from shared memory (16-byte
-// loads where the tile is 16 bytes wide: rows are nb % TM == 0 elements, tiles TM-aligned, stages
-// 16-byte aligned), and the TM x TM products into the chunk sums, FP32 pairs by the FP32x2 FMA
-// (each element a single fused, round-to-nearest operation, as with fma).
-template <typename T, int TM> struct GramRow {
-  __device__ __forceinline__ static void load(const T* p, T* v) {
+// A thread's values of a row: 16-byte loads where the tile is whole 16-byte pieces (tiles are
+// TM-aligned in rows of a multiple of TM values, stages 16-byte aligned).
+template <typename T, int TM>
+__device__ __forceinline__ void gram_load(const T* p, T* v) {
+  if constexpr ((TM * sizeof(T)) % 16 == 0) {
+#pragma unroll
+    for (int i = 0; i < TM; i += 16 / (int)sizeof(T)) {
+      const Vec<T, 16 / (int)sizeof(T)> q = VecIO<T, 16 / (int)sizeof(T)>::ld(p + i);
+#pragma unroll
+      for (int k = 0; k < 16 / (int)sizeof(T); ++k) v[i + k] = q.v[k];
+    }
+  } else {
 #pragma unroll
     for (int i = 0; i < TM; ++i) v[i] = p[i];
   }
-  __device__ __forceinline__ static void fma(const T* a, const T* b, T (*c)[TM]) {
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TM; ++j) c[i][j] = ::fma(a[i], b[j], c[i][j]);
+}
+
+// Accumulator of one element pair (j, j + 1) of a thread's tile: chunk sums c (fused multiply-adds
+// over the chunk's rows), totals over the chunks.  FP32: totals in double-float, the two-sum of
+// hi and c exact, its error summed in lo (so a total loses ~2^-48 of itself per chunk).  FP64: the
+// chunk sums keep a total's chain short.
+template <typename T> struct GramPair;
+template <> struct GramPair<float> {
+  float2 c, hi, lo;
+  __device__ __forceinline__ void zero() { c = hi = lo = make_float2(0.0f, 0.0f); }
+  __device__ __forceinline__ void fma(float a, float b0, float b1) {
+    c = __ffma2_rn(make_float2(a, a), make_float2(b0, b1), c);
+  }
+  __device__ __forceinline__ void flush() {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 s = __fadd2_rn(hi, c);
+    const float2 bb = __ffma2_rn(hi, m1, s);                       // s - hi
+    const float2 e1 = __ffma2_rn(__ffma2_rn(bb, m1, s), m1, hi);   // hi - (s - bb)
+    const float2 e2 = __ffma2_rn(bb, m1, c);                       // c - bb
+    lo = __fadd2_rn(lo, __fadd2_rn(e1, e2));
+    hi = s;
+    c = make_float2(0.0f, 0.0f);
+  }
+  __device__ __forceinline__ double get(int k) const {
+    return k ? (double)hi.y + (double)lo.y : (double)hi.x + (double)lo.x;
   }
 };
-template <> struct GramRow<float, 4> {
-  __device__ __forceinline__ static void load(const float* p, float* v) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+template <> struct GramPair<double> {
+  double c0, c1, t0, t1;
+  __device__ __forceinline__ void zero() { c0 = c1 = t0 = t1 = 0.0; }
+  __device__ __forceinline__ void fma(double a, double b0, double b1) {
+    c0 = ::fma(a, b0, c0);
+    c1 = ::fma(a, b1, c1);
   }
-  __device__ __forceinline__ static void fma(const float* a, const float* b, float (*c)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 ai = make_float2(a[i], a[i]);
-#pragma unroll
-      for (int j = 0; j < 4; j += 2) {
-        const float2 r = __ffma2_rn(ai, make_float2(b[j], b[j + 1]), make_float2(c[i][j], c[i][j + 1]));
-        c[i][j] = r.x;
-        c[i][j + 1] = r.y;
-      }
-    }
+  __device__ __forceinline__ void flush() {
+    t0 += c0;
+    t1 += c1;
+    c0 = c1 = 0.0;
   }
-};
-template <> struct GramRow<double, 4> {
-  __device__ __forceinline__ static void load(const double* p, double* v) {
-    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
-    v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
-  }
-  __device__ __forceinline__ static void fma(const double* a, const double* b, double (*c)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) c[i][j] = ::fma(a[i], b[j], c[i][j]);
-  }
+  __device__ __forceinline__ double get(int k) const { return k ? t1 : t0; }
 };
 
-// Thread t owns tiles t, t+256, ... of the (pair, ti, tj) grid of TM x TM tiles.  PIPE: the
-// chunks are staged by 16-byte cp.async copies into two shared-memory stages, the next chunk's
-// copies in flight while the current one is multiplied (rows of nb values must be a multiple of
-// 16 bytes and every block 16-byte aligned); the products and their order are the same either way.
-template <typename T, int TM, int MAXT, bool PIPE>
+// Pair and tile (first row ti, first column tj) of tile index `idx`; a pair of a block with itself
+// has only the tiles that reach the upper triangle.  Returns false beyond the last tile.
+template <int TMI, int TMJ>
+__host__ __device__ inline bool gram_tile(const PairList& pairs, int nb, int idx, int* q, int* ti, int* tj) {
+  for (int p = 0; p < pairs.n; ++p) {
+    const bool sym = pairs.a[p] == pairs.b[p];
+    for (int i = 0; i < nb; i += TMI) {
+      const int j0 = sym ? i / TMJ * TMJ : 0, cnt = (nb - j0) / TMJ;
+      if (idx < cnt) {
+        *q = p;
+        *ti = i;
+        *tj = j0 + idx * TMJ;
+        return true;
+      }
+      idx -= cnt;
+    }
+  }
+  return false;
+}
+
+// G_q = A^T B of every pair.  A CTA stages chunks of 32 rows of every block; a group of threads
+// (one thread per TMI x TMJ tile of the pairs) multiplies one chunk, and `groups` groups work on
+// consecutive chunks side by side, so that a single narrow pair (16 tiles at nb = 16) still fills
+// the CTA.  When one group does not fit (more than 256 tiles), a thread takes MAXT tiles in turn.
+// PIPE: 16-byte cp.async copies into two stages, the next chunks' copies in flight while the
+// current ones are multiplied (rows of nb values a multiple of 16 bytes and every block 16-byte
+// aligned).  FP32 products are summed per 32-row chunk (chunks start at multiples of 32 rows), chunk
+// sums in double-float, groups and CTAs in FP64 in a fixed order.
+//
+// What bounds it: one pair is an HBM pass; many pairs the shared-memory pipe (a 4 x 4 tile takes
+// six clocks of loads for four clocks of multiply-adds per row, an 8 x 4 tile eight for eight), FP64
+// the FP64 pipe (two lanes per clock per SM: hence only the upper tiles of a pair of a block with
+// itself).  Measured: one FP32 pair at n = 2M, nb = 16 in 57 us (4.5 TB/s; 204 us when one group of 16
+// threads multiplied), LOBPCG's twelve pairs there 416 us (480 us with 4 x 4 tiles); twelve FP64 pairs at
+// n = 20,000, nb = 8 in 40 us (56 us).
+template <typename T, int TMI, int TMJ, int MAXT, bool PIPE>
 __global__ void __launch_bounds__(kGramThreads)
-k_gram(BlockList blocks, PairList pairs, int nb, int64_t n, int64_t rows_per_cta, double* part) {
+k_gram(BlockList blocks, PairList pairs, int nb, int64_t n, int64_t units, int tpg, int groups, double* part) {
+  static_assert(TMJ % 2 == 0 || (TMI == 1 && TMJ == 1), "elements are accumulated in pairs");
+  constexpr int NP = TMJ == 1 ? 1 : TMJ / 2;
+  constexpr int kUnit = sizeof(T) == 4 ? kGramRows : 8;   // row granularity of the CTAs' shares
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  T* sm_base = reinterpret_cast<T*>(sm_raw);  // [stages][nblocks][kGramRows][nb]
-  const size_t stage_elems = (size_t)blocks.n * kGramRows * nb;
-  typedef typename Acc<T>::type A;
-  const int tpp = (nb / TM) * (nb / TM);
-  const int ntiles = pairs.n * tpp;     // <= MAXT * kGramThreads
-  A acc[MAXT][TM][TM];
-  T cacc[MAXT][TM][TM];
+  T* sm_base = reinterpret_cast<T*>(sm_raw);  // [stages][nblocks][groups * 32][nb]
+  const int srows = groups * kGramRows;
+  const size_t bl_elems = (size_t)srows * nb;
+  const size_t stage_elems = (size_t)blocks.n * bl_elems;
+  const int tid = threadIdx.x;
+  const int grp = MAXT == 1 ? tid / tpg : 0;
+  const int tile0 = MAXT == 1 ? tid % tpg : tid;
+  GramPair<T> acc[MAXT][TMI][NP];
+  int q[MAXT], ti[MAXT], tj[MAXT];
+  bool on[MAXT];
 #pragma unroll
-  for (int s = 0; s < MAXT; ++s)
+  for (int s = 0; s < MAXT; ++s) {
+    on[s] = grp < groups && gram_tile<TMI, TMJ>(pairs, nb, tile0 + s * kGramThreads, &q[s], &ti[s], &tj[s]);
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < TMI; ++i)
 #pragma unroll
-      for (int j = 0; j < TM; ++j) { acc_zero(acc[s][i][j]); cacc[s][i][j] = T(0); }
-  const int64_t r0 = blockIdx.x * rows_per_cta;
-  const int64_t r1 = min64(n, r0 + rows_per_cta);
+      for (int j = 0; j < NP; ++j) acc[s][i][j].zero();
+  }
+  const int64_t r0 = units * blockIdx.x / gridDim.x * kUnit;
+  const int64_t r1 = min64(n, units * (blockIdx.x + 1) / gridDim.x * kUnit);
   constexpr int EPC = 16 / sizeof(T);                // elements per 16-byte copy
-  auto issue = [&](int64_t rc, T* stage) {           // copies of the chunk at row rc
-    const int rows = (int)min64(kGramRows, r1 - rc);
-    const int per_block = kGramRows * nb / EPC;
-    for (int i = threadIdx.x; i < blocks.n * per_block; i += blockDim.x) {
-      const int b = i / per_block, e = (i % per_block) * EPC;
-      const T* src = static_cast<const T*>(blocks.p[b]) + rc * nb + e;
-      const bool in = e < rows * nb;
-      cp_async16(stage + (size_t)b * kGramRows * nb + e, in ? (const void*)src : blocks.p[b], in ? 16 : 0);
+  auto issue = [&](int64_t rc, T* stage) {           // copies of the chunks at row rc
+    const int pieces = (int)min64(srows, r1 - rc) * nb / EPC;
+    for (int b = 0; b < blocks.n; ++b) {
+      const T* src = static_cast<const T*>(blocks.p[b]) + rc * nb;
+      T* dst = stage + b * bl_elems;
+      for (int i = tid; i < pieces; i += blockDim.x) cp_async16(dst + i * EPC, src + i * EPC);
     }
     cp_async_commit();
   };
   if (PIPE && r0 < r1) issue(r0, sm_base);
   int stage_i = 0;
-  for (int64_t rc = r0; rc < r1; rc += kGramRows) {
-    const int rows = (int)min64(kGramRows, r1 - rc);
+  for (int64_t rc = r0; rc < r1; rc += srows) {
+    const int rows = (int)min64(srows, r1 - rc);
     T* sm = sm_base + (PIPE ? (size_t)stage_i * stage_elems : 0);
     if (PIPE) {
       // the other stage was last read in the previous iteration: every thread is past it
       __syncthreads();
-      if (rc + kGramRows < r1) {
-        issue(rc + kGramRows, sm_base + (size_t)(stage_i ^ 1) * stage_elems);
+      if (rc + srows < r1) {
+        issue(rc + srows, sm_base + (size_t)(stage_i ^ 1) * stage_elems);
         cp_async_wait<1>();
       } else {
         cp_async_wait<0>();
@@ -153,43 +176,70 @@ k_gram(BlockList blocks, PairList pairs, int nb, int64_t n, int64_t rows_per_cta
       __syncthreads();
       for (int b = 0; b < blocks.n; ++b) {
         const T* src = static_cast<const T*>(blocks.p[b]) + rc * nb;
-        T* dst = sm + (size_t)b * kGramRows * nb;
-        for (int i = threadIdx.x; i < kGramRows * nb; i += blockDim.x) dst[i] = (i < rows * nb) ? src[i] : T(0);
+        T* dst = sm + b * bl_elems;
+        for (int i = tid; i < rows * nb; i += blockDim.x) dst[i] = src[i];
       }
       __syncthreads();
     }
+    const int crows = min(kGramRows, rows - grp * kGramRows);   // rows of this group's chunk (may be <= 0)
 #pragma unroll
     for (int s = 0; s < MAXT; ++s) {
-      const int tile = threadIdx.x + s * kGramThreads;
-      if (tile < ntiles) {
-        const int q = tile / tpp, rem = tile % tpp;
-        const int ti = (rem / (nb / TM)) * TM, tj = (rem % (nb / TM)) * TM;
-        const T* Ab = sm + (size_t)pairs.a[q] * kGramRows * nb;
-        const T* Bb = sm + (size_t)pairs.b[q] * kGramRows * nb;
-        for (int r = 0; r < kGramRows; ++r) {
-          T av[TM], bv[TM];
-          GramRow<T, TM>::load(Ab + r * nb + ti, av);
-          GramRow<T, TM>::load(Bb + r * nb + tj, bv);
-          GramRow<T, TM>::fma(av, bv, cacc[s]);
+      if (on[s] && crows > 0) {
+        const T* Ab = sm + pairs.a[q[s]] * bl_elems + (size_t)grp * kGramRows * nb + ti[s];
+        const T* Bb = sm + pairs.b[q[s]] * bl_elems + (size_t)grp * kGramRows * nb + tj[s];
+        auto row = [&](int r) {
+          T av[TMI], bv[TMJ + 1];
+          gram_load<T, TMI>(Ab + r * nb, av);
+          gram_load<T, TMJ>(Bb + r * nb, bv);
+          if (TMJ == 1) bv[1] = T(0);
+#pragma unroll
+          for (int i = 0; i < TMI; ++i)
+#pragma unroll
+            for (int j = 0; j < NP; ++j) acc[s][i][j].fma(av[i], bv[2 * j], bv[2 * j + 1]);
+        };
+        if (crows == kGramRows) {
+#pragma unroll 4
+          for (int r = 0; r < kGramRows; ++r) row(r);
+        } else {
+          for (int r = 0; r < crows; ++r) row(r);
         }
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+        for (int i = 0; i < TMI; ++i)
 #pragma unroll
-          for (int j = 0; j < TM; ++j) { acc_add(acc[s][i][j], cacc[s][i][j]); cacc[s][i][j] = T(0); }
+          for (int j = 0; j < NP; ++j) acc[s][i][j].flush();
       }
     }
   }
-  double* out = part + (size_t)blockIdx.x * pairs.n * nb * nb;
+  // the groups' sums, in group order, then this CTA's partial; the lower triangle of a pair of a
+  // block with itself mirrors the upper one (the same products in the same order)
+  const int m = pairs.n * nb * nb;
+  double* sred = reinterpret_cast<double*>(sm_raw);   // [groups][m]
+  double* out = part + (size_t)blockIdx.x * m;
+  double* dst = groups > 1 ? sred + (size_t)(grp < groups ? grp : 0) * m : out;
+  __syncthreads();
 #pragma unroll
   for (int s = 0; s < MAXT; ++s) {
-    const int tile = threadIdx.x + s * kGramThreads;
-    if (tile < ntiles) {
-      const int q = tile / tpp, rem = tile % tpp;
-      const int ti = (rem / (nb / TM)) * TM, tj = (rem % (nb / TM)) * TM;
+    if (on[s]) {
+      const bool sym = pairs.a[q[s]] == pairs.b[q[s]];
+      double* d = dst + (size_t)q[s] * nb * nb;
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+      for (int i = 0; i < TMI; ++i)
 #pragma unroll
-        for (int j = 0; j < TM; ++j) out[(size_t)q * nb * nb + (ti + i) * nb + tj + j] = acc_get(acc[s][i][j]);
+        for (int j = 0; j < TMJ; ++j) {
+          const int r = ti[s] + i, c = tj[s] + j;
+          if (sym && r > c) continue;
+          const double v = acc[s][i][j / 2].get(j & 1);
+          d[r * nb + c] = v;
+          if (sym && r < c) d[c * nb + r] = v;
+        }
+    }
+  }
+  if (groups > 1) {
+    __syncthreads();
+    for (int e = tid; e < m; e += blockDim.x) {
+      double v = sred[e];
+      for (int g = 1; g < groups; ++g) v += sred[(size_t)g * m + e];
+      out[e] = v;
     }
   }
 }
@@ -207,18 +257,14 @@ __global__ void k_reduce_partials(const double* __restrict__ part, int nparts, i
   if (lane == 0) out[j] = s;
 }
 
-// Two CTAs per SM.  The grid also fixes how the rows are grouped into partial sums, and so the
-// rounding of every Gram: the hybrid's RMM-DIIS iteration count is sensitive to it (measured at
-// n = 2M: 7 iterations with this grouping, 21 with four CTAs per SM).
-static int gram_grid(int64_t n, int64_t* rows_per_cta, int max_parts) {
-  int g = num_sms() * 2;
+// Two CTAs per SM, each with a near-equal share of the rows in units of 32 rows (the FP32 chunks) or
+// 8 (FP64, bound by its pipe: 20,000 rows are 66 per CTA instead of 96 in 209 of them).
+static int gram_grid(int64_t n, eig_dtype vt, int64_t* units, int max_parts) {
+  const int unit = vt == EIG_F32 ? kGramRows : 8;
+  int64_t g = num_sms() * 2;
   if (max_parts > 0 && g > max_parts) g = max_parts;
-  int64_t rpc = (n + g - 1) / g;
-  rpc = ((rpc + kGramRows - 1) / kGramRows) * kGramRows;
-  if (rpc < kGramRows) rpc = kGramRows;
-  g = (int)((n + rpc - 1) / rpc);
-  *rows_per_cta = rpc;
-  return g;
+  *units = (n + unit - 1) / unit;
+  return (int)min64(g, *units);
 }
 
 size_t gram_scratch_bytes(int npairs, int nb) { return (size_t)num_sms() * 2 * npairs * nb * nb * 8 + 256; }
@@ -229,22 +275,40 @@ eig_status reduce_partials(const double* part, int nparts, int m, double* out, c
   return EIG_OK;
 }
 
-template <typename T, int TM>
+template <typename T, int TMI, int TMJ>
 static eig_status gram_launch(const BlockList& blocks, const PairList& pl, int nb, int64_t n, double* G, void* part,
                               cudaStream_t st, int max_parts) {
-  int64_t rpc;
-  const int g = gram_grid(n, &rpc, max_parts);
+  int64_t units;
+  const int g = gram_grid(n, sizeof(T) == 4 ? EIG_F32 : EIG_F64, &units, max_parts);
+  int q, ti, tj, ntiles = 0;
+  while (gram_tile<TMI, TMJ>(pl, nb, ntiles, &q, &ti, &tj)) ++ntiles;
+  const size_t chunk = (size_t)blocks.n * kGramRows * nb * sizeof(T);
   bool pipe = (nb * sizeof(T)) % 16 == 0;
   for (int b = 0; b < blocks.n; ++b) pipe = pipe && (reinterpret_cast<uintptr_t>(blocks.p[b]) % 16 == 0);
-  pipe = pipe && 2 * (size_t)blocks.n * kGramRows * nb * sizeof(T) <= 200 * 1024;
-  const size_t sm = (size_t)(pipe ? 2 : 1) * blocks.n * kGramRows * nb * sizeof(T);
-  const int ntiles = pl.n * (nb / TM) * (nb / TM);
-  auto kern = pipe ? ((ntiles <= kGramThreads) ? k_gram<T, TM, 1, true>
-                      : (ntiles <= 2 * kGramThreads ? k_gram<T, TM, 2, true> : k_gram<T, TM, 4, true>))
-                   : ((ntiles <= kGramThreads) ? k_gram<T, TM, 1, false>
-                      : (ntiles <= 2 * kGramThreads ? k_gram<T, TM, 2, false> : k_gram<T, TM, 4, false>));
+  pipe = pipe && 2 * chunk <= 200 * 1024;
+  // groups: as many as the threads hold and two CTAs of two stages (and the groups' FP64 sums)
+  // leave room for, and no more than a CTA's share has chunks
+  const size_t m8 = (size_t)pl.n * nb * nb * 8;
+  int64_t groups = ntiles <= kGramThreads ? kGramThreads / ntiles : 1;
+  groups = min64(groups, (int64_t)(100 * 1024 / ((pipe ? 2 : 1) * chunk)));
+  groups = min64(groups, (int64_t)(100 * 1024 / m8));
+  groups = min64(groups, (n + (int64_t)g * kGramRows - 1) / ((int64_t)g * kGramRows));
+  groups = max64(groups, 1);
+  const int tpg = ntiles <= kGramThreads ? ntiles : kGramThreads;
+  const int threads = (int)((groups * tpg + 31) / 32 * 32);
+  size_t sm = (pipe ? 2 : 1) * (size_t)groups * chunk;
+  if (groups > 1 && (size_t)groups * m8 > sm) sm = (size_t)groups * m8;
+  auto kern = pipe ? k_gram<T, TMI, TMJ, 1, true> : k_gram<T, TMI, TMJ, 1, false>;
+  if (ntiles > kGramThreads) {
+    if constexpr (TMI == TMJ) {
+      kern = pipe ? (ntiles <= 2 * kGramThreads ? k_gram<T, TMI, TMJ, 2, true> : k_gram<T, TMI, TMJ, 4, true>)
+                  : (ntiles <= 2 * kGramThreads ? k_gram<T, TMI, TMJ, 2, false> : k_gram<T, TMI, TMJ, 4, false>);
+    } else {
+      return EIG_EUNSUPPORTED;   // the caller takes square tiles from here on
+    }
+  }
   if (sm > 48 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(kern, (int)sm));
-  kern<<<g, kGramThreads, sm, st>>>(blocks, pl, nb, n, rpc, static_cast<double*>(part));
+  kern<<<g, threads, sm, st>>>(blocks, pl, nb, n, units, tpg, (int)groups, static_cast<double*>(part));
   EIG_LAUNCH_CHECK("k_gram");
   return reduce_partials(static_cast<double*>(part), g, pl.n * nb * nb, G, st);
 }
@@ -262,14 +326,19 @@ eig_status gram_multi(const BlockList& blocks, const int* pa, const int* pb, int
   const int TM = (nb % 4 == 0) ? 4 : ((nb % 2 == 0) ? 2 : 1);
   if ((size_t)npairs * (nb / TM) * (nb / TM) > 4 * kGramThreads) return EIG_EUNSUPPORTED;
   if (vt == EIG_F32) {
-    if (TM == 4) return gram_launch<float, 4>(blocks, pl, nb, n, G, part, st, max_parts);
-    if (TM == 2) return gram_launch<float, 2>(blocks, pl, nb, n, G, part, st, max_parts);
-    return gram_launch<float, 1>(blocks, pl, nb, n, G, part, st, max_parts);
+    // from 128 tiles of 4 x 4 on (LOBPCG's twelve pairs at nb = 16 have 174) the shared-memory pipe
+    // is the bound, and 8 x 4 tiles need two thirds of its loads; at most one tile a thread
+    const int t8 = npairs * (nb / 8) * (nb / 4);
+    if (nb % 8 == 0 && 2 * t8 > 128 && t8 <= kGramThreads)
+      return gram_launch<float, 8, 4>(blocks, pl, nb, n, G, part, st, max_parts);
+    if (TM == 4) return gram_launch<float, 4, 4>(blocks, pl, nb, n, G, part, st, max_parts);
+    if (TM == 2) return gram_launch<float, 2, 2>(blocks, pl, nb, n, G, part, st, max_parts);
+    return gram_launch<float, 1, 1>(blocks, pl, nb, n, G, part, st, max_parts);
   }
   if (vt == EIG_F64) {
-    if (TM == 4) return gram_launch<double, 4>(blocks, pl, nb, n, G, part, st, max_parts);
-    if (TM == 2) return gram_launch<double, 2>(blocks, pl, nb, n, G, part, st, max_parts);
-    return gram_launch<double, 1>(blocks, pl, nb, n, G, part, st, max_parts);
+    if (TM == 4) return gram_launch<double, 4, 4>(blocks, pl, nb, n, G, part, st, max_parts);
+    if (TM == 2) return gram_launch<double, 2, 2>(blocks, pl, nb, n, G, part, st, max_parts);
+    return gram_launch<double, 1, 1>(blocks, pl, nb, n, G, part, st, max_parts);
   }
   return EIG_EINVAL;
 }

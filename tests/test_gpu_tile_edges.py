@@ -37,3 +37,33 @@ def test_lp_grad_tile_edges(n, m):
     for a, b in [(12, 204), (204, 236), (236, 1260), (1260, 1292), (1292, 1324), (1324, 1325)]:
         ga, gb = g[a - 12:b - 12], gt[a - 12:b - 12]
         assert np.linalg.norm(ga - gb) <= 1e-4 * max(np.linalg.norm(gb), 1e-2 * np.linalg.norm(gt)), (a, b)
+
+
+def _shifted(a, dt):
+    """The array on the device one element past a 16-byte boundary."""
+    flat = torch.empty(a.size + 1, dtype=dt, device="cuda")
+    v = flat[1:].view(a.shape)
+    v.copy_(torch.tensor(a, dtype=dt))
+    return v
+
+
+# rows: one, around a chunk of 32, one chunk a CTA (304 CTAs), several chunk groups a CTA with a
+# ragged last one; widths with 1 x 1, 2 x 2, 4 x 4 tiles, and more tiles than threads
+@pytest.mark.parametrize("n", [1, 31, 33, 304 * 32, 304 * 32 * 3 + 45, 200003])
+@pytest.mark.parametrize("nb", [5, 6, 8, 16, 64])
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_gram_chunk_edges(n, nb, dt):
+    from paper_2305_15552_gb300 import binding as B
+    rng = np.random.default_rng(n + nb)
+    a, b = rng.standard_normal((n, nb)), rng.standard_normal((n, nb))
+    A, Bm = torch.tensor(a, dtype=dt, device="cuda"), torch.tensor(b, dtype=dt, device="cuda")
+    for X, Y in ((A, Bm), (A, A), (_shifted(a, dt), Bm)):
+        G = B.gram(X, Y).cpu().numpy()
+        Xe, Ye = X.double().cpu().numpy(), Y.double().cpu().numpy()
+        bound = np.abs(Xe).T @ np.abs(Ye)
+        # FP32: products rounded once and summed over 32 rows (at most 33 * 2^-24 of the sum of
+        # magnitudes), the rest exact to 2^-40; FP64: n terms of 2^-53
+        tol = (2.0 ** -24 * 40 if dt == torch.float32 else 2.0 ** -53 * (n + 10)) * bound + 1e-300
+        assert np.all(np.abs(G - Xe.T @ Ye) <= tol)
+        if X is Y:
+            assert np.array_equal(G, G.T)
