@@ -21,59 +21,55 @@ struct AsyncScratch {
   ~AsyncScratch() { if (p) cudaFreeAsync(p, st); }
 };
 
-__global__ void k_small_matmul(const double* __restrict__ A, const double* __restrict__ B, int k,
-                               double* __restrict__ C) {
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-    const int i = e / k, j = e % k;
-    double s = 0.0;
-    for (int l = 0; l < k; ++l) s += A[i * k + l] * B[l * k + j];
-    C[e] = s;
-  }
-}
-
 // CholQR2 of X (in place); X2 (optional, same shape) receives the same right factors, so that
-// X2 <- X2 R^{-1} (used for H Q = (H Y) R^{-1}).
+// X2 <- X2 R^{-1} (used for H Q = (H Y) R^{-1}).  Everything is enqueued at once: a pass whose
+// Cholesky factor breaks down leaves X as it is (its apply skips on the device flag; the next
+// pass then meets the same Gram and breaks down too), and the flags are read once at the end.
 eig_status cholqr2_impl2(void* X, void* X2, int64_t n, int k, eig_dtype vt, double* R, cudaStream_t st) {
   AsyncScratch sc(st);
   const size_t gb = gram_scratch_bytes(1, k);
-  EIG_TRY(sc.get(gb + 4 * (size_t)k * k * 8 + small_chol_inv_work_bytes(k) + 256 * 4));
+  EIG_TRY(sc.get(gb + 3 * (size_t)k * k * 8 + small_chol_inv_work_bytes(k) + 256 * 4));
   unsigned char* base = (unsigned char*)sc.p;
   double* part = (double*)base;
   double* G = (double*)(base + gb);
   double* R1 = G + k * k;
   double* Ri = R1 + k * k;
-  double* R2 = Ri + k * k;
-  double* work = R2 + k * k;
+  double* work = Ri + k * k;
   int* info = (int*)((unsigned char*)work + small_chol_inv_work_bytes(k));
-  int hinfo = 0;
+  AsyncScratch tmp(st);   // only for block widths or alignments that rows_apply does not take
   for (int pass = 0; pass < 2; ++pass) {
     BlockList bl;
     bl.n = 1;
     bl.p[0] = X;
     const int pa = 0, pb = 0;
     EIG_TRY(gram_multi(bl, &pa, &pb, 1, k, n, vt, G, part, st));
-    EIG_TRY(small_chol_inv(G, k, 1e-14, pass == 0 ? R1 : R2, Ri, nullptr, work, info, st));
-    EIG_CUDA_TRY(cudaMemcpyAsync(&hinfo, info, 4, cudaMemcpyDeviceToHost, st));
-    EIG_CUDA_TRY(cudaStreamSynchronize(st));
-    if (hinfo != SMALL_OK) return EIG_EBREAKDOWN;
-    // X <- X R^{-1}: block_apply cannot work in place; stage through a copy
-    void* tmp = nullptr;
-    EIG_CUDA_TRY(cudaMallocAsync(&tmp, (size_t)n * k * dtype_size(vt), st));
+    // the second pass writes R = R2 R1 straight away
+    EIG_TRY(small_chol_inv(G, k, 1e-14, pass == 0 ? R1 : R, Ri, nullptr, pass == 0 ? nullptr : R1, work, info + pass,
+                           st));
     for (int which = 0; which < (X2 ? 2 : 1); ++which) {
       void* Xw = which ? X2 : X;
-      EIG_CUDA_TRY(cudaMemcpyAsync(tmp, Xw, (size_t)n * k * dtype_size(vt), cudaMemcpyDeviceToDevice, st));
-      BlockList in;
-      in.n = 1;
-      in.p[0] = tmp;
-      eig_status s = block_apply(in, k, Ri, k, Xw, 0.0, n, vt, st);
-      if (s != EIG_OK) { cudaFreeAsync(tmp, st); return s; }
+      eig_status s = rows_apply(Xw, k, Ri, Xw, n, vt, info + pass, st);
+      if (s == EIG_EUNSUPPORTED) {
+        // block_apply cannot work in place and does not know the flag: stage through a copy, and
+        // wait for the flag first
+        int hinfo = 0;
+        EIG_CUDA_TRY(cudaMemcpyAsync(&hinfo, info + pass, 4, cudaMemcpyDeviceToHost, st));
+        EIG_CUDA_TRY(cudaStreamSynchronize(st));
+        if (hinfo != SMALL_OK) return EIG_EBREAKDOWN;
+        if (!tmp.p) EIG_TRY(tmp.get((size_t)n * k * dtype_size(vt)));
+        EIG_CUDA_TRY(cudaMemcpyAsync(tmp.p, Xw, (size_t)n * k * dtype_size(vt), cudaMemcpyDeviceToDevice, st));
+        BlockList in;
+        in.n = 1;
+        in.p[0] = tmp.p;
+        s = block_apply(in, k, Ri, k, Xw, 0.0, n, vt, st);
+      }
+      EIG_TRY(s);
     }
-    cudaFreeAsync(tmp, st);
   }
-  k_small_matmul<<<1, 256, 0, st>>>(R2, R1, k, R);
-  EIG_LAUNCH_CHECK("k_small_matmul");
+  int hinfo[2] = {0, 0};
+  EIG_CUDA_TRY(cudaMemcpyAsync(hinfo, info, 8, cudaMemcpyDeviceToHost, st));
   EIG_CUDA_TRY(cudaStreamSynchronize(st));
-  return EIG_OK;
+  return hinfo[0] == SMALL_OK && hinfo[1] == SMALL_OK ? EIG_OK : EIG_EBREAKDOWN;
 }
 
 }  // namespace eig

@@ -26,6 +26,12 @@ eig_status gram_multi(const BlockList& blocks, const int* pa, const int* pb, int
 eig_status block_apply(const BlockList& in, int nb, const double* M, int m, void* Out, double beta, int64_t n,
                        eig_dtype vt, cudaStream_t st);
 
+// Out = In M, M nb x nb (FP64), block width nb 8 or 16, In and Out 16-byte aligned and possibly the
+// same block; EIG_EUNSUPPORTED otherwise (use block_apply).  skip (device int, may be null): Out is
+// left untouched when *skip != 0.
+eig_status rows_apply(const void* In, int nb, const double* M, void* Out, int64_t n, eig_dtype vt, const int* skip,
+                      cudaStream_t st);
+
 // Elementwise conversions / copies of n*k elements.
 eig_status convert(const void* src, eig_dtype st_, void* dst, eig_dtype dt_, int64_t count, cudaStream_t st);
 

@@ -1055,8 +1055,9 @@ eig_status small_rr(const double* A, const double* G, int k, int nb, double piv_
 // ---------------------------------------------------------------------------------------
 template <typename S, bool SM>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_chol_inv(const double* G, int k, double piv_tol, double* R,
-                                                                     double* Rinv, float* Rinv32, double* gwork,
-                                                                     int* info, int) {
+                                                                     double* Rinv, float* Rinv32,
+                                                                     const double* Rprev, double* gwork, int* info,
+                                                                     int) {
   __shared__ S red[33];
   extern __shared__ __align__(128) unsigned char s_dyn[];
   S* g = SM ? reinterpret_cast<S*>(s_dyn) : reinterpret_cast<S*>(gwork);  // k*k: the factor L
@@ -1080,7 +1081,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_chol_inv(const doubl
   trsm_lower(g, k, rd, li, k, k);
   for (int idx = tid; idx < k * k; idx += nt) {
     const int i = idx / k, l = idx % k;
-    R[idx] = (l >= i) ? (double)g[l * k + i] : 0.0;
+    double r = (l >= i) ? (double)g[l * k + i] : 0.0;
+    if (Rprev) {   // R Rprev, both upper triangular
+      r = 0.0;
+      for (int q = i; q <= l; ++q) r += (double)g[q * k + i] * Rprev[q * k + l];
+    }
+    R[idx] = r;
     const double ri = (l >= i) ? (double)li[l * k + i] : 0.0;
     Rinv[idx] = ri;
     if (Rinv32) Rinv32[idx] = (float)ri;
@@ -1088,14 +1094,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_chol_inv(const doubl
   if (tid == 0) *info = SMALL_OK;
 }
 
-eig_status small_chol_inv(const double* G, int k, double piv_tol, double* R, double* Rinv, float* Rinv32, void* work,
-                          int* info, cudaStream_t st) {
+eig_status small_chol_inv(const double* G, int k, double piv_tol, double* R, double* Rinv, float* Rinv32,
+                          const double* Rprev, void* work, int* info, cudaStream_t st) {
   if (k < 1 || k > kSmallMax * 4) return EIG_EINVAL;
   const int sm = smem_launch_bytes(k_small_chol_inv<SmallR, true>, small_chol_inv_work_bytes(k));
   if (sm > 0)
-    k_small_chol_inv<SmallR, true><<<1, kSmallThreads, sm, st>>>(G, k, piv_tol, R, Rinv, Rinv32, (double*)work, info, 1);
+    k_small_chol_inv<SmallR, true><<<1, kSmallThreads, sm, st>>>(G, k, piv_tol, R, Rinv, Rinv32, Rprev, (double*)work,
+                                                                      info, 1);
   else
-    k_small_chol_inv<SmallR, false><<<1, kSmallThreads, 0, st>>>(G, k, piv_tol, R, Rinv, Rinv32, (double*)work, info, 0);
+    k_small_chol_inv<SmallR, false><<<1, kSmallThreads, 0, st>>>(G, k, piv_tol, R, Rinv, Rinv32, Rprev, (double*)work,
+                                                                      info, 0);
   EIG_LAUNCH_CHECK("k_small_chol_inv");
   return EIG_OK;
 }

@@ -37,10 +37,11 @@ eig_status small_rr(const double* A, const double* G, int k, int nb, double piv_
                     float* C32, void* work, int* info, cudaStream_t st, int pivoted = 0);
 
 // CholQR factor: G = R^T R (upper R) and Rinv = R^{-1}, k x k; info = SMALL_BREAKDOWN when a
-// squared pivot falls below piv_tol * max diag(G).  Rinv32: optional float copy.
+// squared pivot falls below piv_tol * max diag(G).  Rinv32: optional float copy.  Rprev (optional,
+// upper triangular): R receives the product of the factor with it.
 // work: small_chol_inv_work_bytes(k) bytes of device scratch.
 size_t small_chol_inv_work_bytes(int k);
 eig_status small_chol_inv(const double* G, int k, double piv_tol, double* R, double* Rinv, float* Rinv32,
-                          void* work, int* info, cudaStream_t st);
+                          const double* Rprev, void* work, int* info, cudaStream_t st);
 
 }  // namespace eig

@@ -67,3 +67,37 @@ def test_gram_chunk_edges(n, nb, dt):
         assert np.all(np.abs(G - Xe.T @ Ye) <= tol)
         if X is Y:
             assert np.array_equal(G, G.T)
+
+
+# rows: fewer than one warp pass, around the 256 / 512 rows of a CTA pass, ragged; widths with the
+# in-place apply (8, 16) and without; a block off the 16-byte boundary
+@pytest.mark.parametrize("n", [16, 31, 257, 1025, 608 * 512 + 7])
+@pytest.mark.parametrize("k", [5, 8, 16])
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+@pytest.mark.parametrize("shift", [False, True])
+def test_cholqr2_row_edges(n, k, dt, shift):
+    from paper_2305_15552_gb300 import binding as B
+    x = np.random.default_rng(n + k).standard_normal((n, k)) * np.logspace(0, -1, k)
+    X = _shifted(x, dt) if shift else torch.tensor(x, dtype=dt, device="cuda")
+    Xe = X.double().cpu().numpy()
+    Q, R = B.cholqr2(X)
+    Q, R = Q.double().cpu().numpy(), R.cpu().numpy()
+    eps = 2.0 ** -24 if dt == torch.float32 else 2.0 ** -53
+    # the second pass works on a basis orthonormal to ~cond^2 eps: Q^T Q - I is a few rounding errors
+    # of k-term rows and of the Gram; Q R reproduces X to two k-term products per pass
+    assert np.abs(Q.T @ Q - np.eye(k)).max() < 40 * k * eps
+    assert np.abs(Q @ R - Xe).max() < 40 * k * eps * np.abs(Xe).max()
+    assert np.array_equal(R, np.triu(R))
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_cholqr2_breakdown_leaves_block(dt):
+    from paper_2305_15552_gb300 import binding as B
+    x = np.random.default_rng(3).standard_normal((3000, 8))
+    x[:, 5] = 0.0                        # a pivot of exactly zero
+    X = torch.tensor(x, dtype=dt, device="cuda")
+    Y = X.clone()
+    with pytest.raises(B.EigError) as e:
+        B.cholqr2(X)
+    assert e.value.status == B.EIG_EBREAKDOWN
+    assert torch.equal(X, Y)
