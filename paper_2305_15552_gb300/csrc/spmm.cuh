@@ -54,11 +54,13 @@ struct SpmmPlan {
   DevBuf scratch;      // transposed partial products, n_slots * C * nb * sizeof(T)
   // mirrored copy of H (both triangles; gather-only kernel): per row block of 256 rows, its
   // column tiles (64 columns) cut into panels of at most 24 tiles; per panel the rows ranked by
-  // entry count, lane l of warp w taking the row of rank 32 w + l; per (panel, warp) a stream
+  // entry count (within m_groups groups of consecutive rows), lane l of warp w taking the row of
+  // rank 32 w + l; per (panel, warp) a stream
   // of blocks of 32 lanes x 8 steps of (uint16 panel-local column, value), padded with
   // zero-valued entries on zero rows
   bool mirrored = false;
   int64_t m_npan = 0, m_nblk = 0, m_full_nnz = 0;
+  int m_pr = 0, m_groups = 1;        // staged X rows of the widest panel; row groups (CTAs) per row block
   DevBuf m_rbp;                      // int32[nRB+1]: panels of row block I
   DevBuf m_pt0, m_pnt;               // int32[m_npan]: first tile (into m_tcol) and tile count
   DevBuf m_tcol;                     // int32: column block of each tile of the mirrored matrix

@@ -15,13 +15,18 @@
 //     column tiles, the rows are ranked by their entry count and warp w's lane l takes the
 //     row of rank 32 w + l; the warp steps through its longest row's count, shorter rows
 //     padded with zero-valued entries (a few percent);
+//   * a matrix with fewer row blocks than SMs ranks its rows within two halves of the row block
+//     instead, each half's warps a CTA of their own (row_groups);
 //   * each step, lane l gathers its entry's whole X row in 16-byte pieces, starting at a
 //     lane-dependent piece, and the entries are ordered so that lane l reads a row of class
 //     (l + step) mod 8 (X row index mod 8): the 8 lanes of every shared-memory phase then hit
 //     distinct banks for any nb;
 //   * the entries (uint16 panel-local column + value) stream from HBM straight into registers,
 //     several 8-step blocks ahead, bypassing L1 and evicted first from L2; each lane loads
-//     only its own entries (16 + 32 bytes per block in FP32), so nothing is loaded twice;
+//     only its own entries (16 + 32 bytes per block in FP32), a warp's 16-byte pieces side by side,
+//     so that nothing is loaded twice and a load is four full wavefronts (with a lane's 32 bytes of
+//     values side by side instead, n = 2M, 400 nonzeros a row took 1.80 ms at nb = 16 and 1.09 at
+//     nb = 8, against 1.74 and 1.02);
 //   * X: the X rows of the row block's column tiles (64 rows each) are staged in shared
 //     memory by bulk copies (TMA) in panels of at most 24 tiles, evicted last from L2; a row
 //     block whose tiles do not fit takes several panels, its rows' partial sums added in Y
@@ -46,8 +51,8 @@ constexpr int kW = 8;                    // warps per CTA; warp w takes the rows
 constexpr int kRW = kMR / kW;            // rows per warp
 constexpr int kBS = 8;                   // steps per streamed block
 constexpr int kBE = 32 * kBS;            // entries per block (32 lanes)
-constexpr int kPT = 24;                  // tiles per panel at most
-constexpr int kPR = kPT * kMC;           // staged X rows per panel; 8 zero rows follow
+constexpr int kPT = 24;                  // tiles per panel at most (<= 32: one lane stages one tile)
+constexpr int kPR = kPT * kMC;           // staged X rows per panel at most; 8 zero rows follow
 constexpr int kL2 = 6;                   // streamed blocks prefetched into L2 ahead of use
 
 // ---------------------------------------------------------------------------------------
@@ -215,9 +220,10 @@ __global__ void k_rs_counts(int64_t n, const int64_t* __restrict__ fptr, const i
   }
 }
 
-// CTA per panel: the panel's 256 rows ranked by entry count (descending, ties by row), so that
-// each warp's 32 lanes take rows of near-equal length; steps of each warp = its longest row.
-__global__ void __launch_bounds__(kMR) k_rs_rank(const uint16_t* __restrict__ cnt, uint8_t* __restrict__ perm,
+// CTA per panel: the panel's 256 rows ranked by entry count (descending, ties by row) within each
+// group of `gr` consecutive rows (256: one group), so that each warp's 32 lanes take rows of
+// near-equal length; steps of each warp = its longest row.
+__global__ void __launch_bounds__(kMR) k_rs_rank(const uint16_t* __restrict__ cnt, int gr, uint8_t* __restrict__ perm,
                                                  int32_t* __restrict__ steps) {
   __shared__ uint16_t c[kMR];
   const int64_t p = blockIdx.x;
@@ -225,8 +231,9 @@ __global__ void __launch_bounds__(kMR) k_rs_rank(const uint16_t* __restrict__ cn
   c[t] = cnt[p * kMR + t];
   __syncthreads();
   const int mine = c[t];
-  int rank = 0;
-  for (int u = 0; u < kMR; ++u) {
+  const int g0 = t / gr * gr;
+  int rank = g0;
+  for (int u = g0; u < g0 + gr; ++u) {
     const int o = c[u];
     rank += (o > mine) || (o == mine && u < t);
   }
@@ -234,14 +241,23 @@ __global__ void __launch_bounds__(kMR) k_rs_rank(const uint16_t* __restrict__ cn
   if (rank % kRW == 0) steps[p * kW + rank / kRW] = mine;
 }
 
+// Values of a streamed block: 16-byte pieces (kEpp consecutive steps of one lane), piece-major, so
+// that a warp's load of one piece per lane is contiguous.  Columns: [lane][step] (16 bytes a lane).
+template <typename V> struct BlkPiece { static constexpr int kEpp = 16 / (int)sizeof(V); };
+template <typename V>
+__device__ __forceinline__ int64_t blk_value_at(int lane, int step) {
+  constexpr int E = BlkPiece<V>::kEpp;
+  return (int64_t)(step / E) * 32 * E + lane * E + step % E;
+}
+
 // Every stream position starts as padding: value 0 and the zero row of the class its lane
-// wants at that step.  Block layout: [lane][step], 32 lanes x 8 steps.
+// wants at that step.
 template <typename VS>
-__global__ void k_rs_pads(int64_t nent, uint16_t* __restrict__ bcol, VS* __restrict__ bval) {
+__global__ void k_rs_pads(int64_t nent, int pr, uint16_t* __restrict__ bcol, VS* __restrict__ bval) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= nent) return;
   const int lane = (int)((e % kBE) / kBS), k = (int)(e % kBS);
-  bcol[e] = (uint16_t)(kPR + ((lane + k) & 7));
+  bcol[e] = (uint16_t)(pr + ((lane + k) & 7));
   bval[e] = VS(0);
 }
 
@@ -291,7 +307,7 @@ __global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ 
                                                     const int32_t* __restrict__ pan_rb, const int32_t* __restrict__ pt0,
                                                     const int32_t* __restrict__ pnt, const int32_t* __restrict__ tcol,
                                                     const uint8_t* __restrict__ perm, const int64_t* __restrict__ sboff,
-                                                    uint16_t* __restrict__ sc, uint16_t* __restrict__ bcol,
+                                                    int pr, uint16_t* __restrict__ sc, uint16_t* __restrict__ bcol,
                                                     V* __restrict__ bval) {
   static_assert(kBS == 8 && (kBS * sizeof(V)) % 16 == 0, "a lane's block is whole 16-byte pieces");
   __shared__ int32_t s_tc[kPT];
@@ -383,7 +399,7 @@ __global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ 
         cc = (uint32_t)(lo * kMC + (col - J * kMC));
         v = fval[e];
       } else {  // padding, as k_rs_pads writes it
-        cc = (uint32_t)(kPR + ((lane + k) & 7));
+        cc = (uint32_t)(pr + ((lane + k) & 7));
         v = V(0);
       }
       cw[j >> 1] |= cc << (16 * (j & 1));
@@ -392,11 +408,17 @@ __global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ 
     const int64_t at = (blk0 + b) * kBE + lane * kBS;
     *reinterpret_cast<uint4*>(bcol + at) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
     const uint4* src = reinterpret_cast<const uint4*>(vv);
-    uint4* dst = reinterpret_cast<uint4*>(bval + at);
 #pragma unroll
-    for (int u = 0; u < (int)(kBS * sizeof(V) / 16); ++u) dst[u] = src[u];
+    for (int u = 0; u < (int)(kBS * sizeof(V) / 16); ++u)
+      *reinterpret_cast<uint4*>(bval + (blk0 + b) * kBE + blk_value_at<V>(lane, u * BlkPiece<V>::kEpp)) = src[u];
   }
 }
+
+// Row groups of a row block.  With fewer row blocks than SMs each half of a row block is a CTA of
+// its own: ranking within a half pads one to two percent more and X is staged twice, but n = 20,000
+// (79 row blocks, 100 nonzeros a row, FP32) takes 22.7 instead of 28.2 us at nb = 8 and 25.5 instead
+// of 32.8 at nb = 16; at 196 row blocks it no longer gains, at 391 it loses.
+int row_groups(int64_t nRB) { return nRB < num_sms() ? 2 : 1; }
 
 template <typename V>
 eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* tile_cb, int64_t n_up_tiles,
@@ -467,6 +489,9 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   }
   const int64_t npan = rbp[nRB];
   P->m_npan = npan;
+  // staged rows: those of the widest panel
+  P->m_pr = std::max(1, *std::max_element(pnt.begin(), pnt.end())) * kMC;
+  P->m_groups = row_groups(nRB);
   EIG_TRY(P->m_rbp.reserve((nRB + 1) * 4));
   EIG_TRY(P->m_pt0.reserve(npan * 4));
   EIG_TRY(P->m_pnt.reserve(npan * 4));
@@ -493,7 +518,8 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   EIG_LAUNCH_CHECK("k_rs_counts");
   EIG_TRY(P->m_perm.reserve(npan * kMR));
   EIG_TRY(steps.reserve(npan * kW * 4));
-  k_rs_rank<<<(unsigned)npan, kMR, 0, st>>>(cntp.as<uint16_t>(), P->m_perm.as<uint8_t>(), steps.as<int32_t>());
+  k_rs_rank<<<(unsigned)npan, kMR, 0, st>>>(cntp.as<uint16_t>(), kMR / P->m_groups, P->m_perm.as<uint8_t>(),
+                                            steps.as<int32_t>());
   EIG_LAUNCH_CHECK("k_rs_rank");
   std::vector<int32_t> h_steps(npan * kW);
   std::vector<int64_t> sboff(npan * kW + 1, 0);
@@ -510,7 +536,8 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   const int64_t nent = std::max<int64_t>(nblk, 1) * kBE;
   EIG_TRY(P->m_bcol.reserve(nent * 2));
   EIG_TRY(P->m_bval.reserve(nent * sizeof(V)));
-  k_rs_pads<V><<<(unsigned)((nent + tb - 1) / tb), tb, 0, st>>>(nent, P->m_bcol.as<uint16_t>(), P->m_bval.as<V>());
+  k_rs_pads<V><<<(unsigned)((nent + tb - 1) / tb), tb, 0, st>>>(nent, P->m_pr, P->m_bcol.as<uint16_t>(),
+                                                                P->m_bval.as<V>());
   EIG_LAUNCH_CHECK("k_rs_pads");
   if (npan > 0) {
     DevBuf sc;  // class buckets, at each row segment's positions in the mirrored CSR
@@ -518,7 +545,7 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
     k_rs_scatter<V><<<(unsigned)npan, kMR, 0, st>>>(
         fptr.as<int64_t>(), fcol.as<int32_t>(), fval.as<V>(), n, d_pan_rb.as<int32_t>(), P->m_pt0.as<int32_t>(),
         P->m_pnt.as<int32_t>(), P->m_tcol.as<int32_t>(), P->m_perm.as<uint8_t>(), P->m_sboff.as<int64_t>(),
-        sc.as<uint16_t>(), P->m_bcol.as<uint16_t>(), P->m_bval.as<V>());
+        P->m_pr, sc.as<uint16_t>(), P->m_bcol.as<uint16_t>(), P->m_bval.as<V>());
     EIG_LAUNCH_CHECK("k_rs_scatter");
   }
   EIG_CUDA_TRY(cudaStreamSynchronize(st));  // temporaries go out of scope
@@ -539,6 +566,7 @@ struct RsArgs {
   const int64_t* sboff;
   const uint16_t* bcol;
   const void* bval;
+  int pr;        // staged rows of the widest panel; the zero rows follow them
   int* err;
 };
 
@@ -584,7 +612,7 @@ template <typename T, typename V, int NB> struct RsShape {
   static constexpr int EPC = LDB / ES;        // elements per piece
   // lanes of a phase reading the same bank-line offset class get distinct pieces
   static constexpr int ROTDIV = NCH >= 8 ? 1 : 8 / NCH;
-  static constexpr size_t XBYTES = (size_t)(kPR + 8) * RBY;
+  static constexpr size_t XBYTES = (size_t)(kPR + 8) * RBY;   // at most
   static constexpr int MINB0 = (int)(233472 / (XBYTES + 1024 + 128));
   // register budget: up to 4 CTAs per SM for rows of <= 16 bytes, 3 for 32, else (and for
   // FP64 values, whose blocks take twice the registers) 2
@@ -774,11 +802,41 @@ template <> struct Stage<double, true> {
   }
 };
 
-// Row block I of one product.  Y (and X, Qp) rows have stride ld elements; the product covers
-// elements [col0, col0 + NB).
+// Double-float staging of whole rows (ld == NB >= 2): a thread converts 16-byte pieces (two elements,
+// the accumulator's piece layout), eight loads in flight.  One element at a time each panel waited
+// for ~30 round trips to L2: 3.21 ms instead of 2.95 at n = 2M (400 nonzeros a row), nb = 8.
+template <int NB>
+__device__ __forceinline__ void stage_df_rows(unsigned char* xs, const double* __restrict__ X, const int32_t* tcol,
+                                              int npt, int64_t n) {
+  constexpr int PPR = NB / 2, U = 8;   // pieces per row, loads in flight
+  const int total = npt * kMC * PPR;
+  for (int i0 = threadIdx.x; i0 < total; i0 += U * blockDim.x) {
+    double2 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * blockDim.x;
+      x[u] = make_double2(0.0, 0.0);
+      if (i < total) {
+        const int64_t row = (int64_t)tcol[i / (kMC * PPR)] * kMC + i / PPR % kMC;
+        if (row < n) x[u] = __ldg(reinterpret_cast<const double2*>(X + row * NB) + i % PPR);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * blockDim.x;
+      if (i >= total) break;
+      const float h0 = __double2float_rn(x[u].x), h1 = __double2float_rn(x[u].y);
+      reinterpret_cast<float4*>(xs)[i] = make_float4(h0, h1, __double2float_rn(x[u].x - (double)h0),
+                                                     __double2float_rn(x[u].y - (double)h1));
+    }
+  }
+}
+
+// Warps [w0, w0 + blockDim.x / 32) of row block I of one product.  Y (and X, Qp) rows have stride ld
+// elements; the product covers elements [col0, col0 + NB).
 template <typename T, typename V, int NB, bool CHEB>
 __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __restrict__ X, T* __restrict__ Y, int ld,
-                                                 int col0, int xj_bulk, const MirrorEpi& epi, int64_t I) {
+                                                 int col0, int xj_bulk, const MirrorEpi& epi, int64_t I, int w0) {
   typedef RsShape<T, V, NB> Sh;
   constexpr bool DF = Sh::DF;
   constexpr int RBY = Sh::RBY, LDB = Sh::LDB, NCH = Sh::NCH, EPC = Sh::EPC, PF = Sh::PF, VW = Sh::VW;
@@ -789,15 +847,17 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
   typedef typename Acc::OT OT;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* xs = smem;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Sh::XBYTES);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)(a.pr + 8) * RBY);
   __shared__ int s_abort;
 
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // warps of a scheduler (every fourth) take a long and a short stream: 0 1 2 3 7 6 5 4
+  const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+  const int w = w0 + (wi < 4 ? wi : 11 - wi);
   const int64_t r0 = I * kMR;
   const int p0 = a.rbp[I], p1 = a.rbp[I + 1];
 
   // zero rows (one per class) for the padding entries; never overwritten by staging
-  for (int i = tid; i < 8 * RBY / 4; i += kW * 32) reinterpret_cast<uint32_t*>(xs + (size_t)kPR * RBY)[i] = 0u;
+  for (int i = tid; i < 8 * RBY / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(xs + (size_t)a.pr * RBY)[i] = 0u;
   if (tid == 0) {
     s_abort = 0;
     mbar_init(bar, 1);
@@ -820,39 +880,27 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
     __syncthreads();  // the previous panel's gathers are done
     const int t0 = a.pt0[p], npt = a.pnt[p];
     if (xj_bulk) {
-      if (tid == 0 && npt > 0) {
-        uint32_t tot = 0;
-        for (int t = 0; t < npt; ++t) {
-          const int64_t cb0 = (int64_t)a.tcol[t0 + t] * kMC;
-          tot += (uint32_t)(min64(kMC, a.n - cb0) * RBY);
-        }
-        mbar_arrive_expect_tx(bar, tot);
-        for (int t = 0; t < npt; ++t) {
-          const int64_t cb0 = (int64_t)a.tcol[t0 + t] * kMC;
-          const uint32_t bytes = (uint32_t)(min64(kMC, a.n - cb0) * RBY);
-          tma_load_1d_hint(xs + (size_t)t * kMC * RBY, X + cb0 * NB, bytes, bar, pol_keep);
-        }
+      // one bulk copy per tile, issued by one lane each (at most kPT <= 32 tiles)
+      if (tid < 32 && npt > 0) {
+        const int64_t cb0 = lane < npt ? (int64_t)a.tcol[t0 + lane] * kMC : 0;
+        const uint32_t bytes = lane < npt ? (uint32_t)(min64(kMC, a.n - cb0) * RBY) : 0u;
+        const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
+        if (lane == 0) mbar_arrive_expect_tx(bar, tot);
+        __syncwarp();
+        if (lane < npt) tma_load_1d_hint(xs + (size_t)lane * kMC * RBY, X + cb0 * NB, bytes, bar, pol_keep);
       }
-      if (npt > 0) {
-        if (!mbar_wait_bounded(bar, xphase)) {
-          atomicOr(a.err, 1);
-          s_abort = 1;
-        }
-        __syncthreads();
-        if (s_abort) break;
-        xphase ^= 1u;
-      }
+    } else if (DF && NB >= 2 && ld == NB) {
+      if constexpr (DF && NB >= 2) stage_df_rows<NB>(xs, X, a.tcol + t0, npt, a.n);
     } else {
-      for (int64_t i = tid; i < (int64_t)npt * kMC * NB; i += kW * 32) {
+      for (int64_t i = tid; i < (int64_t)npt * kMC * NB; i += blockDim.x) {
         const int t = (int)(i / (kMC * NB));
         const int rr = (int)((i / NB) % kMC), e = (int)(i % NB);
         const int64_t row = (int64_t)a.tcol[t0 + t] * kMC + rr;
         if (row < a.n) Stage<T, DF>::put(xs + (size_t)(t * kMC + rr) * RBY, e, NB, X[row * ld + col0 + e]);
       }
-      __syncthreads();
     }
 
-    // this lane's row and the warp's stream
+    // this lane's row and the warp's stream; its first blocks load while X is staged
     const int64_t r = r0 + a.perm[(int64_t)p * kMR + w * 32 + lane];
     const int L = a.steps[(int64_t)p * kW + w];
     const int64_t b0 = a.sboff[(int64_t)p * kW + w];
@@ -866,7 +914,8 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
       bc[s] = ldg_stream(bcol + e, pol_stream);
 #pragma unroll
       for (int u = 0; u < VW; u += 4) {
-        const uint4 t = ldg_stream(reinterpret_cast<const unsigned char*>(bval + e) + u * 4, pol_stream);
+        const uint4 t = ldg_stream(bval + (b0 + b) * kBE + blk_value_at<VS>(lane, u / 4 * BlkPiece<VS>::kEpp),
+                                   pol_stream);
         bv[s][u] = t.x; bv[s][u + 1] = t.y; bv[s][u + 2] = t.z; bv[s][u + 3] = t.w;
       }
     };
@@ -882,6 +931,19 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
 #pragma unroll
     for (int s = 0; s < PF; ++s)
       if (s < nb) load_blk(s, s);
+    if (xj_bulk) {
+      if (npt > 0) {
+        if (!mbar_wait_bounded(bar, xphase)) {
+          atomicOr(a.err, 1);
+          s_abort = 1;
+        }
+        __syncthreads();
+        if (s_abort) break;
+        xphase ^= 1u;
+      }
+    } else {
+      __syncthreads();
+    }
     for (int b = 0; b < nb; b += PF) {
 #pragma unroll
       for (int s = 0; s < PF; ++s) {
@@ -966,12 +1028,13 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
   }
 }
 
-// One product: CTA = row block.
+// One product: CTA = row block, or one of its row groups.
 template <typename T, typename V, int NB, bool CHEB>
 __global__ void __launch_bounds__(kW * 32, RsShape<T, V, NB>::MINB)
 k_spmm_mirror(const __grid_constant__ RsArgs a, const T* __restrict__ X, T* __restrict__ Y, int ld, int col0,
               int xj_bulk, const __grid_constant__ MirrorEpi epi) {
-  mirror_row_block<T, V, NB, CHEB>(a, X, Y, ld, col0, xj_bulk, epi, blockIdx.x);
+  const int g = kW * 32 / blockDim.x;   // CTAs per row block
+  mirror_row_block<T, V, NB, CHEB>(a, X, Y, ld, col0, xj_bulk, epi, blockIdx.x / g, (int)(blockIdx.x % g) * (kW / g));
 }
 
 // Several products of one shape in one launch over their concatenated row blocks (the
@@ -983,7 +1046,7 @@ k_spmm_mirror_batch(const __grid_constant__ MirrorBatch B) {
   while (j + 1 < B.n && B.cta0[j + 1] <= (int64_t)blockIdx.x) ++j;
   const MirrorJob& J = B.jobs[j];
   mirror_row_block<T, V, NB, CHEB>(J.a, static_cast<const T*>(J.X), static_cast<T*>(J.Y), J.ld, J.col0, J.xj_bulk,
-                                   J.epi, (int64_t)blockIdx.x - B.cta0[j]);
+                                   J.epi, (int64_t)blockIdx.x - B.cta0[j], 0);
 }
 
 }  // namespace
@@ -1068,6 +1131,7 @@ static RsArgs rs_args(SpmmPlan* P) {
   a.sboff = P->m_sboff.as<int64_t>();
   a.bcol = P->m_bcol.as<uint16_t>();
   a.bval = P->m_bval.p;
+  a.pr = P->m_pr;
   a.err = P->err.as<int>();
   return a;
 }
@@ -1085,13 +1149,15 @@ static eig_status rs_launch(SpmmPlan* P, const T* X, T* Y, int ld, int col0, con
   int dev = 0, maxsm = 0;
   EIG_CUDA_TRY(cudaGetDevice(&dev));
   EIG_CUDA_TRY(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const size_t sm = Sh::XBYTES + 16;
+  const size_t sm = (size_t)(P->m_pr + 8) * Sh::RBY + 16;
   if (sm > (size_t)maxsm) return EIG_EUNSUPPORTED;
   const RsArgs a = rs_args(P);
   const int xj_bulk = rs_xj_bulk<T, V, NBK>(X, ld);
   auto kern = k_spmm_mirror<T, V, NBK, CHEB>;
   EIG_CUDA_TRY(::eig::ensure_dyn_smem(kern, (int)sm));
-  kern<<<(unsigned)P->nRB, kW * 32, sm, st>>>(a, X, Y, ld, col0, xj_bulk, epi);
+  // the threads themselves stage double-float X: a whole CTA per row block then
+  const int groups = xj_bulk ? P->m_groups : 1;
+  kern<<<(unsigned)(P->nRB * groups), kW * 32 / groups, sm, st>>>(a, X, Y, ld, col0, xj_bulk, epi);
   EIG_LAUNCH_CHECK(CHEB ? "k_spmm_mirror_cheb" : "k_spmm_mirror");
   return EIG_OK;
 }
@@ -1113,10 +1179,13 @@ eig_status mirror_launch_batch(const SpmmJob* jobs, int count, cudaStream_t st) 
   int dev = 0, maxsm = 0;
   EIG_CUDA_TRY(cudaGetDevice(&dev));
   EIG_CUDA_TRY(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const size_t sm = Sh::XBYTES + 16;
-  if (sm > (size_t)maxsm) return EIG_EUNSUPPORTED;
-  for (int i = 0; i < count; ++i)
+  int pr = 0;
+  for (int i = 0; i < count; ++i) {
     if (!jobs[i].P->mirrored) return EIG_EUNSUPPORTED;
+    pr = std::max(pr, jobs[i].P->m_pr);
+  }
+  const size_t sm = (size_t)(pr + 8) * Sh::RBY + 16;
+  if (sm > (size_t)maxsm) return EIG_EUNSUPPORTED;
   auto kern = k_spmm_mirror_batch<T, V, NBK, CHEB>;
   EIG_CUDA_TRY(::eig::ensure_dyn_smem(kern, (int)sm));
   MirrorBatch B;

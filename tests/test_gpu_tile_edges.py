@@ -101,3 +101,26 @@ def test_cholqr2_breakdown_leaves_block(dt):
         B.cholqr2(X)
     assert e.value.status == B.EIG_EBREAKDOWN
     assert torch.equal(X, Y)
+
+
+# row blocks: one fewer and one more than the 152 SMs' worth at which a row block stops being split
+# into two CTAs (the last one ragged), and a single row block of a few rows
+@pytest.mark.parametrize("n", [40, 151 * 256 + 9, 152 * 256 + 9])
+@pytest.mark.parametrize("val,dt,nb", [("f32", torch.float32, 1), ("f32", torch.float32, 16), ("f32", torch.float64, 8),
+                                       ("bf16", torch.float32, 8), ("bf16", torch.float64, 16), ("f64", torch.float64, 8)])
+def test_spmm_row_group_edges(n, val, dt, nb):
+    import oracle as O
+    from gen import ci_matrix, random_block
+    from paper_2305_15552_gb300 import binding as B
+    H = ci_matrix(n, 40, 64, seed=3, storage=val)
+    X = torch.tensor(random_block(n, nb, seed=4), dtype=dt, device="cuda")
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y = P.spmm(X).double().cpu().numpy()
+    P.close()
+    Xe = X.double().cpu().numpy()
+    Ha = type(H)(n=n, rowptr=H.rowptr, col=H.col, val=np.abs(H.values_f64()), storage="f64")
+    bound = O.sym_upper_matmul(Ha, np.abs(Xe))
+    # rows of at most a few hundred terms: one rounding per multiply-add (FP32, FP64), 2^-44 per
+    # double-float step
+    eps = 2.0 ** -24 if dt == torch.float32 else (2.0 ** -53 if val == "f64" else 2.0 ** -44)
+    assert np.all(np.abs(Y - O.sym_upper_matmul(H, Xe)) <= 300 * eps * bound + 1e-300)
