@@ -69,6 +69,11 @@ struct SpmmPlan {
   DevBuf m_sboff;                    // int64[m_npan * 8 + 1]: first block of each (panel, warp)
   DevBuf m_bcol;                     // uint16[m_nblk * 256]
   DevBuf m_bval;                     // value type [m_nblk * 256]
+  // direct streams (small FP64 matrices, in place of panels): rows ranked over the whole matrix, each
+  // on m_dsplit lanes; m_sboff[w] the first block of warp w, m_bcol the column of H itself
+  bool m_direct = false;
+  int m_dsplit = 1;
+  DevBuf m_drow, m_dlen;             // int32 per slot: row (n: none), entries
   double algorithmic_bytes(int nb, size_t vec_bytes) const;
 };
 

@@ -33,6 +33,9 @@
 //     in panel order.
 // Every sum runs in a fixed order (steps in stream order, panels in order): Y is bitwise
 // reproducible.
+//
+// Small FP64 matrices (FP64 values, n < 65,536: direct_plan) take the streams without row blocks
+// and panels; see k_spmm_direct.
 #include <algorithm>
 #include <vector>
 
@@ -420,6 +423,96 @@ __global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ 
 // of 32.8 at nb = 16; at 196 row blocks it no longer gains, at 391 it loses.
 int row_groups(int64_t nRB) { return nRB < num_sms() ? 2 : 1; }
 
+// ---------------------------------------------------------------------------------------
+// Plan: direct streams (no row blocks, no panels)
+// ---------------------------------------------------------------------------------------
+// FP64 products run at the FP64 pipe's rate (one warp multiply-add per 64 clocks per scheduler), so
+// what matters is that every scheduler has the same number of them; with few rows, row blocks of
+// unequal length on unequal numbers of CTAs per SM left the busiest scheduler with 2.6 times the
+// average (n = 20,000, 100 nonzeros a row).  The columns are row indices of X in 16 bits, hence the
+// bound on n; there (65,000 rows, 100 or 400 nonzeros a row) the direct streams still take 0.56 and
+// 0.57 of the panels' time at nb = 8 (100 against 177 us, 385 against 677) and 0.51 to 0.57 at nb = 1.
+bool direct_plan(const SpmmPlan* P) { return P->val_type == EIG_F64 && P->n < 65536; }
+
+// Warp per row: its entries, columns ascending and the diagonal last, dealt to its `split` lanes in
+// turn (slot_of: the row's first slot).
+__global__ void k_direct_fill(int64_t n, int split, const int64_t* __restrict__ fptr, const int32_t* __restrict__ fcol,
+                              const double* __restrict__ fval, const int32_t* __restrict__ slot_of,
+                              const int64_t* __restrict__ sboff, uint16_t* __restrict__ bcol,
+                              double* __restrict__ bval) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (r >= n) return;
+  const int64_t e0 = fptr[r];
+  const int len = (int)(fptr[r + 1] - e0);
+  const int slot = slot_of[r];
+  const int64_t blk0 = sboff[slot >> 5];
+  int before = 0;   // entries left of the diagonal, or len without one
+  for (int q0 = 0; q0 < len; q0 += 32) {
+    const int c = q0 + lane < len ? fcol[e0 + q0 + lane] : INT32_MAX;
+    before += __popc(__ballot_sync(0xffffffffu, (int64_t)c < r));
+  }
+  const bool diag = before < len && (int64_t)fcol[e0 + before] == r;
+  for (int q = lane; q < len; q += 32) {
+    const int i = !diag || q < before ? q : (q == before ? len - 1 : q - 1);
+    const int k = i / split, sl = (slot & 31) + i % split;
+    const int64_t at = (blk0 + k / kBS) * kBE;
+    bcol[at + sl * kBS + k % kBS] = (uint16_t)fcol[e0 + q];
+    bval[at + blk_value_at<double>(sl, k % kBS)] = fval[e0 + q];
+  }
+}
+
+// Rows ranked by length over the whole matrix (descending, ties by row): warp w takes ranks
+// [32 w / split, 32 (w + 1) / split), each row on `split` adjacent lanes.
+eig_status direct_fill(SpmmPlan* P, const std::vector<int64_t>& h_len, const int64_t* fptr, const int32_t* fcol,
+                       const double* fval, cudaStream_t st) {
+  const int64_t n = P->n;
+  // lanes per row: until a block of 8 (two slices) gives eight warps per scheduler
+  int split = 1;
+  while (split < 4 && (n * split + 31) / 32 * 2 < (int64_t)num_sms() * 32) split *= 2;
+  const int64_t nw = (n * split + 31) / 32;
+  int64_t longest = 0;
+  for (int64_t l : h_len) longest = std::max(longest, l);
+  std::vector<int64_t> start(longest + 2, 0);
+  for (int64_t l : h_len) start[longest - l + 1]++;
+  for (int64_t l = 0; l <= longest; ++l) start[l + 1] += start[l];
+  std::vector<int32_t> slot_of(n), row(nw * 32, (int32_t)n), len(nw * 32, 0);
+  for (int64_t r = 0; r < n; ++r) {
+    const int64_t q = start[longest - h_len[r]]++ * split;
+    slot_of[r] = (int32_t)q;
+    for (int j = 0; j < split; ++j) {
+      row[q + j] = (int32_t)r;
+      len[q + j] = (int32_t)((h_len[r] - j + split - 1) / split);
+    }
+  }
+  std::vector<int64_t> sboff(nw + 1, 0);
+  for (int64_t w = 0; w < nw; ++w) sboff[w + 1] = sboff[w] + (len[w * 32] + kBS - 1) / kBS;
+  P->m_dsplit = split;
+  P->m_nblk = sboff[nw];
+  DevBuf d_slot;
+  EIG_TRY(d_slot.reserve(n * 4));
+  EIG_TRY(P->m_drow.reserve(nw * 32 * 4));
+  EIG_TRY(P->m_dlen.reserve(nw * 32 * 4));
+  EIG_TRY(P->m_sboff.reserve((nw + 1) * 8));
+  EIG_CUDA_TRY(cudaMemcpyAsync(d_slot.p, slot_of.data(), n * 4, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(P->m_drow.p, row.data(), nw * 32 * 4, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(P->m_dlen.p, len.data(), nw * 32 * 4, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(P->m_sboff.p, sboff.data(), (nw + 1) * 8, cudaMemcpyHostToDevice, st));
+  const int64_t nent = std::max<int64_t>(P->m_nblk, 1) * kBE;
+  EIG_TRY(P->m_bcol.reserve(nent * 2));
+  EIG_TRY(P->m_bval.reserve(nent * 8));
+  // padding: zero values, which the kernel multiplies by zeros of its own (its lengths bound the loads)
+  EIG_CUDA_TRY(cudaMemsetAsync(P->m_bcol.p, 0, nent * 2, st));
+  EIG_CUDA_TRY(cudaMemsetAsync(P->m_bval.p, 0, nent * 8, st));
+  k_direct_fill<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, split, fptr, fcol, fval, d_slot.as<int32_t>(),
+                                                                  P->m_sboff.as<int64_t>(), P->m_bcol.as<uint16_t>(),
+                                                                  P->m_bval.as<double>());
+  EIG_LAUNCH_CHECK("k_direct_fill");
+  EIG_CUDA_TRY(cudaStreamSynchronize(st));  // temporaries go out of scope
+  P->m_direct = true;
+  return EIG_OK;
+}
+
 template <typename V>
 eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* tile_cb, int64_t n_up_tiles,
                           const int64_t* jt_ptr, const int32_t* jt_tile, cudaStream_t st) {
@@ -465,6 +558,9 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   cnt.release();
   off.release();
   lower.release();
+  if constexpr (sizeof(V) == 8) {
+    if (direct_plan(P)) return direct_fill(P, h_len, fptr.as<int64_t>(), fcol.as<int32_t>(), fval.as<V>(), st);
+  }
   // 3. tiles of the mirrored matrix per row block, cut into panels of at most kPT tiles
   //    (balanced: a row block of t tiles takes ceil(t / kPT) panels of near-equal size; a row
   //    block without tiles still gets one empty panel so that its rows are written)
@@ -1049,6 +1145,127 @@ k_spmm_mirror_batch(const __grid_constant__ MirrorBatch B) {
                                    J.epi, (int64_t)blockIdx.x - B.cta0[j], 0);
 }
 
+// Product of a direct plan, FP64: a warp takes 32 lanes' worth of rows (a row on `split` adjacent
+// lanes) and NB <= 4 of the block's columns, gathering its rows of X through L1 and L2 (32 bytes per
+// entry: one sector, one load).
+//
+// What bounds it: the FP64 pipe, and for few rows the longest row's chain of gathers and
+// multiply-adds.  Column slices and split rows multiply the warps, so that the longest group (twice the
+// average) is not the makespan; the launch order pairs long with short ones on an SM: CTAs (four warps,
+// one per scheduler, of near-equal length) come in order of length, and every second round of one CTA
+// per SM in the reverse order.  n = 20,000, 100 nonzeros a row: 41 us at nb = 8 (27 us of FP64
+// multiply-adds), 76 at nb = 16, 12.5 at nb = 1; with row blocks and panels 143, 262 and 38.
+struct DirectArgs {
+  int64_t n;
+  int32_t nw;            // warps' worth of slots
+  int32_t split;         // lanes per row
+  const int32_t* row;    // row of each slot (n: none)
+  const int32_t* len;    // entries of each slot
+  const int64_t* sboff;
+  const uint16_t* bcol;
+  const double* bval;
+  int sms;
+};
+constexpr int kDirectWarps = 4;
+// Four doubles (32 bytes, one sector) in one load.
+__device__ __forceinline__ Vec<double, 4> ld_sector(const double* p) {
+  Vec<double, 4> r;
+  asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+               : "=d"(r.v[0]), "=d"(r.v[1]), "=d"(r.v[2]), "=d"(r.v[3]) : "l"(p));
+  return r;
+}
+
+template <int NB, bool CHEB>
+__global__ void __launch_bounds__(kDirectWarps * 32, 4)
+k_spmm_direct(const __grid_constant__ DirectArgs a, const double* __restrict__ X, double* __restrict__ Y, int ld,
+              int col0, int slices, const __grid_constant__ MirrorEpi epi) {
+  constexpr int VEC = NB >= 2 ? 2 : 1, NCH = NB / VEC;
+  const int lane = threadIdx.x & 31;
+  const int full = (int)gridDim.x / a.sms * a.sms, round = (int)blockIdx.x / a.sms;
+  const int cta = (int)blockIdx.x < full && (round & 1) ? 2 * round * a.sms + a.sms - 1 - (int)blockIdx.x
+                                                        : (int)blockIdx.x;
+  const int task = cta * kDirectWarps + (threadIdx.x >> 5);
+  const int g = task / slices;
+  if (g >= a.nw) return;
+  const int c0 = col0 + task % slices * NB;
+  const int slot = g * 32 + lane;
+  const int len = a.len[slot], L = a.len[g * 32];
+  const int64_t r = a.row[slot];
+  const int64_t b0 = a.sboff[g];
+  const int nb = (L + kBS - 1) / kBS;
+  const uint64_t pol = policy_evict_first();
+  const double* Xc = X + c0;
+  double y[NB];
+#pragma unroll
+  for (int e = 0; e < NB; ++e) y[e] = 0.0;
+  uint4 cw;
+  uint4 vw[4];
+  auto load = [&](int b) {
+    cw = ldg_stream(a.bcol + (b0 + b) * kBE + lane * kBS, pol);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) vw[u] = ldg_stream(a.bval + (b0 + b) * kBE + blk_value_at<double>(lane, 2 * u), pol);
+  };
+  if (nb > 0) load(0);
+  for (int b = 0; b < nb; ++b) {
+    const uint32_t c4[4] = {cw.x, cw.y, cw.z, cw.w};
+    double v[kBS];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[2 * u] = __hiloint2double((int)vw[u].y, (int)vw[u].x);
+      v[2 * u + 1] = __hiloint2double((int)vw[u].w, (int)vw[u].z);
+    }
+    // the block's gathers all start before the first multiply-add; the next block's entries after them
+    Vec<double, VEC> x[kBS][NCH];
+#pragma unroll
+    for (int k = 0; k < kBS; ++k) {
+      const int64_t c = (k & 1) ? (c4[k >> 1] >> 16) : (c4[k >> 1] & 0xFFFFu);
+      if constexpr (NB == 4) {
+        Vec<double, 4> t;
+        t.zero();
+        if (b * kBS + k < len) t = ld_sector(Xc + c * ld);
+        x[k][0].v[0] = t.v[0]; x[k][0].v[1] = t.v[1]; x[k][1].v[0] = t.v[2]; x[k][1].v[1] = t.v[3];
+      } else {
+        x[k][0].zero();
+        if (b * kBS + k < len) x[k][0] = VecIO<double, VEC>::ld(Xc + c * ld);
+      }
+    }
+    if (b + 1 < nb) load(b + 1);
+#pragma unroll
+    for (int k = 0; k < kBS; ++k)
+      if (b * kBS + k < L) {
+#pragma unroll
+        for (int j = 0; j < NCH; ++j)
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) y[j * VEC + e] = fma(v[k], x[k][j].v[e], y[j * VEC + e]);
+      }
+  }
+  for (int o = 1; o < a.split; o <<= 1)
+#pragma unroll
+    for (int e = 0; e < NB; ++e) y[e] += __shfl_xor_sync(0xffffffffu, y[e], o);
+  if (r >= a.n || lane % a.split) return;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    const int jc = c0 + j * VEC;
+    Vec<double, VEC> out;
+    if (CHEB) {
+      const Vec<double, VEC> xv = VecIO<double, VEC>::ld(X + r * ld + jc);
+      Vec<double, VEC> qv;
+      qv.zero();
+      if (!epi.first) qv = VecIO<double, VEC>::ld(static_cast<const double*>(epi.Qp) + r * ld + jc);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        double yv = __dmul_rn(epi.a, __fma_rn(-epi.c, xv.v[e], y[j * VEC + e]));
+        if (!epi.first) yv = __dsub_rn(yv, qv.v[e]);
+        out.v[e] = epi.active[jc + e] ? yv : xv.v[e];
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) out.v[e] = y[j * VEC + e];
+    }
+    VecIO<double, VEC>::st(Y + r * ld + jc, out);
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------
@@ -1162,8 +1379,33 @@ static eig_status rs_launch(SpmmPlan* P, const T* X, T* Y, int ld, int col0, con
   return EIG_OK;
 }
 
+// Columns [col0, col0 + nb) of a direct plan's product, in slices of at most four.
+template <int NB, bool CHEB>
+static eig_status direct_launch(SpmmPlan* P, const double* X, double* Y, int ld, int col0, const MirrorEpi& epi,
+                                cudaStream_t st) {
+  constexpr int NS = NB < 4 ? NB : 4;
+  DirectArgs a;
+  a.n = P->n;
+  a.split = P->m_dsplit;
+  a.nw = (int32_t)((P->n * a.split + 31) / 32);
+  a.row = P->m_drow.as<int32_t>();
+  a.len = P->m_dlen.as<int32_t>();
+  a.sboff = P->m_sboff.as<int64_t>();
+  a.bcol = P->m_bcol.as<uint16_t>();
+  a.bval = P->m_bval.as<double>();
+  a.sms = num_sms();
+  const int tasks = a.nw * (NB / NS);
+  k_spmm_direct<NS, CHEB><<<(unsigned)((tasks + kDirectWarps - 1) / kDirectWarps), kDirectWarps * 32, 0, st>>>(
+      a, X, Y, ld, col0, NB / NS, epi);
+  EIG_LAUNCH_CHECK(CHEB ? "k_spmm_direct_cheb" : "k_spmm_direct");
+  return EIG_OK;
+}
+
 template <typename T, typename V, int NB>
 eig_status mirror_launch(SpmmPlan* P, const T* X, T* Y, cudaStream_t st) {
+  if constexpr (sizeof(V) == 8) {
+    if (P->m_direct) return direct_launch<NB, false>(P, X, Y, NB, 0, MirrorEpi(), st);
+  }
   constexpr int NBK = RsSlice<T, V, NB>::value;
   for (int c0 = 0; c0 < NB; c0 += NBK) EIG_TRY((rs_launch<T, V, NBK, false>(P, X, Y, NB, c0, MirrorEpi(), st)));
   return EIG_OK;
@@ -1238,6 +1480,9 @@ EIG_MIRROR_BATCH_INST(double, float)
 // a decoupled RMM-DIIS vector (Sec. 4.3), summed in the order of the block product's column.
 template <typename T, typename V>
 eig_status mirror_launch_column(SpmmPlan* P, const T* X, T* Y, int ld, int col, cudaStream_t st) {
+  if constexpr (sizeof(V) == 8) {
+    if (P->m_direct) return direct_launch<1, false>(P, X, Y, ld, col, MirrorEpi(), st);
+  }
   return rs_launch<T, V, 1, false>(P, X, Y, ld, col, MirrorEpi(), st);
 }
 
@@ -1251,6 +1496,9 @@ eig_status mirror_launch_cheb(SpmmPlan* P, const T* X, T* Y, const T* Qp, const 
   epi.a = alpha;
   epi.c = c;
   epi.first = first;
+  if constexpr (sizeof(V) == 8) {
+    if (P->m_direct) return direct_launch<NB, true>(P, X, Y, NB, 0, epi, st);
+  }
   constexpr int NBK = RsSlice<T, V, NB>::value;
   for (int c0 = 0; c0 < NB; c0 += NBK) EIG_TRY((rs_launch<T, V, NBK, true>(P, X, Y, NB, c0, epi, st)));
   return EIG_OK;

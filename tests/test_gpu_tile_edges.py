@@ -124,3 +124,37 @@ def test_spmm_row_group_edges(n, val, dt, nb):
     # double-float step
     eps = 2.0 ** -24 if dt == torch.float32 else (2.0 ** -53 if val == "f64" else 2.0 ** -44)
     assert np.all(np.abs(Y - O.sym_upper_matmul(H, Xe)) <= 300 * eps * bound + 1e-300)
+
+
+# direct plans (FP64 values below 65,536 rows): fewer rows than a warp, a ragged last warp, one CTA
+# round of the 152 SMs and a few CTAs more, the last size they take and the first they do not; every
+# width, one column in place, the fused Chebyshev step, empty rows, rows without a diagonal
+@pytest.mark.parametrize("n", [1, 33, 2500, 65535, 65536])
+@pytest.mark.parametrize("nb", [1, 2, 4, 8, 16, 32])
+def test_spmm_direct_edges(n, nb):
+    import oracle as O
+    from gen import ci_matrix, random_block
+    from gen.synth import CSRUpper
+    from paper_2305_15552_gb300 import binding as B
+    H = ci_matrix(n, 30, 64, seed=5, storage="f64")
+    rows = np.repeat(np.arange(n), np.diff(H.rowptr))
+    keep = ~((rows % 7 == 3) & (H.col == rows)) & (rows % 11 != 5) & (H.col % 11 != 5)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(rows[keep], minlength=n), out=rowptr[1:])
+    H = CSRUpper(n=n, rowptr=rowptr, col=H.col[keep], val=H.val[keep], storage="f64")
+    Xe = random_block(n, nb, seed=6)
+    X = torch.tensor(Xe, device="cuda")
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y = P.spmm(X).cpu().numpy()
+    Ha = CSRUpper(n=n, rowptr=H.rowptr, col=H.col, val=np.abs(H.val), storage="f64")
+    Yr, bound = O.sym_upper_matmul(H, Xe), O.sym_upper_matmul(Ha, np.abs(Xe))
+    tol = 300 * 2.0 ** -53 * bound + 1e-300     # one rounding per multiply-add, rows of at most 300
+    assert np.all(np.abs(Y - Yr) <= tol)
+    if nb >= 8:
+        Q = torch.tensor(random_block(n, nb, seed=7), device="cuda")
+        act = torch.tensor([j % 3 != 1 for j in range(nb)], dtype=torch.int32, device="cuda")
+        Z = P.spmm_cheb(X, 0.5, 2.0, Q, act).cpu().numpy()
+        want = np.where(act.cpu().numpy() != 0, 0.5 * (Y - 2.0 * Xe) - Q.cpu().numpy(), Xe)
+        # three roundings of the step on the same H X
+        assert np.all(np.abs(Z - want) <= 4 * 2.0 ** -53 * (np.abs(Y) + 2 * np.abs(Xe) + np.abs(Q.cpu().numpy())))
+    P.close()
