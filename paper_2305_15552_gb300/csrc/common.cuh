@@ -60,19 +60,31 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 inline size_t dtype_size(eig_dtype t) { return t == EIG_F64 ? 8 : (t == EIG_F32 ? 4 : 2); }
 
-// Device buffer owned by the library (cudaMalloc / cudaFree).
+// Device buffer owned by the library (cudaMalloc / cudaFree), or a part of one (borrow).
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
+  bool owned = true;
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
   ~DevBuf() { release(); }
   void release() {
-    if (p) cudaFree(p);
+    if (p && owned) cudaFree(p);
     p = nullptr;
     bytes = 0;
+    owned = true;
   }
+  // Becomes bytes [off, off + b) of `of`, which must outlive it; advances off to the next part.
+  void borrow(const DevBuf& of, size_t b, size_t* off) {
+    release();
+    p = static_cast<unsigned char*>(of.p) + *off;
+    bytes = b;
+    owned = false;
+    *off += part(b);
+  }
+  // Size of a part: parts start on 256-byte boundaries, as allocations do.
+  static size_t part(size_t b) { return (b + 255) & ~size_t(255); }
   // Ensures at least `b` bytes; contents are not preserved when it grows.
   eig_status reserve(size_t b) {
     if (b <= bytes && p) return EIG_OK;

@@ -28,6 +28,7 @@ struct SpmmPlan {
   const int64_t* rowptr = nullptr;
   const int32_t* col = nullptr;
   const void* val = nullptr;
+  DevBuf own;                           // what is known when building starts: the CSR copy, tile_ptr, diag, err
   DevBuf own_rowptr, own_col, own_val;
   // tile lists: tiles of row block I are tile_col[tile_ptr[I] .. tile_ptr[I+1]), ascending J
   int64_t n_tiles = 0, n_slots = 0;
@@ -59,7 +60,8 @@ struct SpmmPlan {
   // of blocks of 32 lanes x 8 steps of (uint16 panel-local column, value), padded with
   // zero-valued entries on zero rows
   bool mirrored = false;
-  int64_t m_npan = 0, m_nblk = 0, m_full_nnz = 0;
+  DevBuf m_own, m_streams;           // the panel arrays; m_bcol and m_bval
+  int64_t m_npan = 0, m_nblk = 0;
   int m_pr = 0, m_groups = 1;        // staged X rows of the widest panel; row groups (CTAs) per row block
   DevBuf m_rbp;                      // int32[nRB+1]: panels of row block I
   DevBuf m_pt0, m_pnt;               // int32[m_npan]: first tile (into m_tcol) and tile count
@@ -79,13 +81,23 @@ struct SpmmPlan {
 
 eig_status spmm_plan_build(SpmmPlan* P, const eig_csr_upper* H, int R, int C, int layout, int copy,
                            cudaStream_t st);
-// Per row block of R rows, the ascending column blocks (of C) in which a sorted CSR has entries.
-eig_status build_tile_lists(int64_t n, int R, int C, const int64_t* rowptr, const int32_t* col, cudaStream_t st,
-                            DevBuf& tile_ptr, DevBuf& tile_col, std::vector<int64_t>& h_ptr,
-                            std::vector<int32_t>& h_col);
-// Builds the mirrored layout from the plan's CSR and tile lists (R = 256, C = 64 only).
+// Temporaries of a plan's construction that depend on n alone.
+struct PlanTemps {
+  DevBuf mem;
+  DevBuf bitmap;                     // nRB x words: tiles of the upper triangle, later of both; an int flag behind
+  DevBuf rb_cnt, rb_ptr;             // int64[nRB], int64[nRB + 1]
+  DevBuf lower, lptr, sums;          // int64[n], [n + 1], and the scan's chunk sums
+  eig_status reserve(int64_t n, int64_t nRB, int64_t words, bool mirror);
+};
+// Per row block, the ascending column blocks set in its row (words_per_rb words) of the bitmap; cnt:
+// device int64[nRB].
+eig_status tile_lists_from_bitmap(int64_t nRB, int64_t words_per_rb, const unsigned* bitmap, int64_t* cnt,
+                                  cudaStream_t st, DevBuf& tile_ptr, DevBuf& tile_col, std::vector<int64_t>& h_ptr,
+                                  std::vector<int32_t>& h_col);
+// Builds the mirrored layout from the plan's CSR and tile lists (R = 256, C = 64 only); the bitmap of
+// the upper tiles becomes that of both triangles.
 eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tptr,
-                                  const std::vector<int32_t>& h_tcol, cudaStream_t st);
+                                  const std::vector<int32_t>& h_tcol, PlanTemps& tmp, cudaStream_t st);
 // Device bytes the mirrored layout needs while it is built (estimate).
 size_t mirror_bytes_estimate(const SpmmPlan* P);
 // Builds the tile-contiguous copy (called by spmm_plan_build).

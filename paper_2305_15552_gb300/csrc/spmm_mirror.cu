@@ -59,61 +59,101 @@ constexpr int kPR = kPT * kMC;           // staged X rows per panel at most; 8 z
 constexpr int kL2 = 6;                   // streamed blocks prefetched into L2 ahead of use
 
 // ---------------------------------------------------------------------------------------
-// Plan: both triangles as a CSR, built from U without sorting and without atomics on values
+// Plan: the strictly lower triangle as a CSR beside the upper one, built from U without sorting and
+// without atomics on values.  A row of H is its row of the lower CSR, then its row of U.
 // ---------------------------------------------------------------------------------------
 
-// Entries of row r with columns in [lo, hi) (rows are sorted): [*a, *b).
-__device__ __forceinline__ void row_segment(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                            int64_t r, int64_t lo, int64_t hi, int64_t* a, int64_t* b) {
-  int64_t L = rowptr[r], H = rowptr[r + 1];
-  const int64_t end = H;
-  while (L < H) {
-    const int64_t m = (L + H) >> 1;
-    if (col[m] < lo) L = m + 1; else H = m;
+// Index of tile column J among the nt <= 32 ascending columns tc, which hold it: slot[J mod 256] names
+// one tile (J < 2^25 in the upper bits, its index in the lower five); where it names another, by search.
+__device__ __forceinline__ int tile_index(const uint32_t* slot, const int32_t* tc, int nt, int32_t J) {
+  const uint32_t x = slot[J & 255];
+  if (x >> 5 == (uint32_t)J) return (int)(x & 31u);
+  int lo = 0;
+  for (int hi = nt - 1; lo < hi;) {
+    const int mid = (lo + hi) >> 1;
+    if (tc[mid] < J) lo = mid + 1; else hi = mid;
   }
-  *a = L;
-  H = end;
-  while (L < H) {
-    const int64_t m = (L + H) >> 1;
-    if (col[m] < hi) L = m + 1; else H = m;
-  }
-  *b = L;
+  return lo;
 }
 
-// Column-major bitmap of the strictly-upper entries of upper tile t (256 rows x 64 columns):
-// bits[j * 8 + w] bit b <=> entry (row 32 w + b, column j).  One thread per row.
-__device__ void tile_bits(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                          int64_t r0, int64_t cb0, unsigned* bits, int64_t* a, int64_t* b) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < kMC * (kMR / 32); i += blockDim.x) bits[i] = 0u;
-  __syncthreads();
-  const int64_t r = r0 + tid;
-  *a = *b = 0;
-  if (r < n) {
-    row_segment(rowptr, col, r, cb0, cb0 + kMC, a, b);
-    for (int64_t k = *a; k < *b; ++k) {
-      const int64_t c = col[k];
-      if (c != r) atomicOr(&bits[(c - cb0) * (kMR / 32) + (tid >> 5)], 1u << (tid & 31));
-    }
-  }
-  __syncthreads();
-}
-
-// Per upper tile: how many strictly-upper entries each of its 64 columns holds.
+// CTA per row block, warp per row (32 rows each), the row block's upper tiles (256 rows x 64 columns) in
+// groups of kCountTiles.  Per tile: seg[t * 256 + row], the offset in its row of the row's first entry
+// in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper entries of each
+// column (integer atomics in shared memory: order independent); the largest total of a tile; and, in the
+// bitmap of the full matrix, the transposed tiles (64 rows of this row block as a column block of the
+// row block that holds the tile's columns).
+constexpr int kCountTiles = 32;
 __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ col,
-                                                       const int32_t* __restrict__ tile_rb,
-                                                       const int32_t* __restrict__ tile_cb,
-                                                       int32_t* __restrict__ cnt) {
-  __shared__ unsigned bits[kMC * (kMR / 32)];
-  const int64_t t = blockIdx.x;
-  int64_t a, b;
-  tile_bits(n, rowptr, col, (int64_t)tile_rb[t] * kMR, (int64_t)tile_cb[t] * kMC, bits, &a, &b);
-  if (threadIdx.x < kMC) {
-    int s = 0;
+                                                       const int64_t* __restrict__ tile_ptr,
+                                                       const int32_t* __restrict__ tile_col, int64_t words_per_rb,
+                                                       int32_t* __restrict__ seg, int32_t* __restrict__ cnt,
+                                                       unsigned* __restrict__ bitmap, int* __restrict__ most) {
+  __shared__ int s_cnt[kCountTiles][kMC];
+  __shared__ int32_t s_tc[kCountTiles];
+  __shared__ uint32_t s_slot[256];          // tile column and index, at the column mod 256 (one of them)
+  __shared__ unsigned s_sub[kCountTiles];   // bit q: the 64 rows q have strictly-upper entries in the tile
+  const int64_t I = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t t0 = tile_ptr[I], t1 = tile_ptr[I + 1];
+  for (int64_t g0 = t0; g0 < t1; g0 += kCountTiles) {
+    const int nt = (int)min64(kCountTiles, t1 - g0);
+    __syncthreads();
+    for (int i = tid; i < kCountTiles * kMC; i += kMR) (&s_cnt[0][0])[i] = 0;
+    if (tid < kCountTiles) {
+      s_tc[tid] = tid < nt ? tile_col[g0 + tid] : INT32_MAX;
+      s_sub[tid] = 0u;
+    }
+    s_slot[tid] = 0xffffffffu;
+    __syncthreads();
+    if (tid < nt) s_slot[s_tc[tid] & 255] = ((uint32_t)s_tc[tid] << 5) | tid;
+    __syncthreads();
+    const int32_t first = s_tc[0], last = s_tc[nt - 1];
+    for (int lr = w; lr < kMR; lr += kW) {
+      const int64_t r = I * kMR + lr;
+      if (r >= n) break;
+      const int64_t e0 = rowptr[r], e1 = rowptr[r + 1];
+      int32_t before = -1;   // tile column of the entry before the chunk
+      bool past = false;
+      for (int64_t q0 = e0; q0 < e1 && !past; q0 += 128) {
+        int32_t cs[4];
 #pragma unroll
-    for (int w = 0; w < kMR / 32; ++w) s += __popc(bits[threadIdx.x * (kMR / 32) + w]);
-    cnt[t * kMC + threadIdx.x] = s;
+        for (int u = 0; u < 4; ++u) cs[u] = q0 + 32 * u + lane < e1 ? col[q0 + 32 * u + lane] : INT32_MAX;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int32_t c = cs[u], J = c / kMC;
+          const int32_t up = __shfl_up_sync(0xffffffffu, J, 1);
+          if (c != INT32_MAX && J >= first && J <= last) {
+            const int lo = tile_index(s_slot, s_tc, nt, J);
+            if ((lane == 0 ? before : up) != J) {
+              seg[(g0 + lo) * kMR + lr] = (int32_t)(q0 + 32 * u + lane - e0);
+              // a row whose only entry here is its diagonal has nothing strictly upper, but the tile
+              // then belongs to this row block already
+              if ((s_sub[lo] >> (lr / kMC) & 1u) == 0u) atomicOr(&s_sub[lo], 1u << (lr / kMC));
+            }
+            if ((int64_t)c != r) atomicAdd(&s_cnt[lo][c - J * kMC], 1);
+          }
+          before = __shfl_sync(0xffffffffu, J, 31);
+        }
+        past = before > last;   // also after the row's end (INT32_MAX)
+      }
+    }
+    __syncthreads();
+    for (int t = w; t < nt; t += kW) {
+      int total = 0;
+#pragma unroll
+      for (int h = 0; h < kMC; h += 32) {
+        const int x = s_cnt[t][h + lane];
+        cnt[(g0 + t) * kMC + h + lane] = x;
+        total += x;
+      }
+      total = warp_sum(total);
+      if (lane == 0 && total) atomicMax(most, total);
+      if (lane < 4 && (s_sub[t] >> lane & 1u)) {
+        const int64_t Q = I * (kMR / kMC) + lane;
+        atomicOr(bitmap + s_tc[t] / (kMR / kMC) * words_per_rb + (Q >> 5), 1u << (Q & 31));
+      }
+    }
   }
 }
 
@@ -135,59 +175,193 @@ __global__ void k_mir_coloffsets(int64_t n, const int64_t* __restrict__ jt_ptr, 
   lower[c] = run;
 }
 
-// Row lengths of the mirrored matrix.
-__global__ void k_mir_rowlen(int64_t n, const int64_t* __restrict__ rowptr, const int64_t* __restrict__ lower,
-                             int64_t* __restrict__ len) {
-  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r < n) len[r] = lower[r] + rowptr[r + 1] - rowptr[r];
+// Exclusive prefix sums in three passes over chunks of kScanChunk values: chunk sums, the sums'
+// own prefix (one CTA), the chunks.
+constexpr int kScanThreads = 256, kScanChunk = 4 * kScanThreads;
+
+__device__ __forceinline__ int64_t scan_block(int64_t v, int64_t* total) {   // exclusive, over the CTA
+  __shared__ int64_t s_w[kScanThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int64_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t t = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += t;
+  }
+  __syncthreads();   // the previous use of s_w is over
+  if (lane == 31) s_w[w] = x;
+  __syncthreads();
+  int64_t base = 0, all = 0;
+#pragma unroll
+  for (int i = 0; i < kScanThreads / 32; ++i) {
+    if (i < w) base += s_w[i];
+    all += s_w[i];
+  }
+  *total = all;
+  return base + x - v;
+}
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int64_t* __restrict__ v, int64_t n,
+                                                            int64_t* __restrict__ sums) {
+  int64_t s = 0, total;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t e = blockIdx.x * (int64_t)kScanChunk + i * kScanThreads + threadIdx.x;
+    if (e < n) s += v[e];
+  }
+  scan_block(s, &total);
+  if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(kScanThreads) k_scan_tops(int64_t* __restrict__ sums, int64_t m) {
+  int64_t run = 0;
+  for (int64_t b = 0; b < m; b += kScanThreads) {
+    const int64_t e = b + threadIdx.x;
+    int64_t total;
+    const int64_t x = scan_block(e < m ? sums[e] : 0, &total);
+    if (e < m) sums[e] = run + x;
+    run += total;
+  }
+}
+// out[0..n]: out[n] is the total.
+__global__ void __launch_bounds__(kScanThreads) k_scan_chunks(const int64_t* __restrict__ v, int64_t n,
+                                                              const int64_t* __restrict__ sums,
+                                                              int64_t* __restrict__ out) {
+  int64_t run = sums[blockIdx.x];
+  for (int i = 0; i < 4; ++i) {
+    const int64_t e = blockIdx.x * (int64_t)kScanChunk + i * kScanThreads + threadIdx.x;
+    int64_t total;
+    const int64_t x = scan_block(e < n ? v[e] : 0, &total);
+    if (e < n) out[e] = run + x;
+    if (e == n - 1) out[n] = run + x + v[e];
+    run += total;
+  }
+}
+static eig_status exclusive_scan(const int64_t* v, int64_t n, int64_t* out, int64_t* sums, cudaStream_t st) {
+  const int64_t m = (n + kScanChunk - 1) / kScanChunk;
+  k_scan_sums<<<(unsigned)m, kScanThreads, 0, st>>>(v, n, sums);
+  EIG_LAUNCH_CHECK("k_scan_sums");
+  k_scan_tops<<<1, kScanThreads, 0, st>>>(sums, m);
+  EIG_LAUNCH_CHECK("k_scan_tops");
+  k_scan_chunks<<<(unsigned)m, kScanThreads, 0, st>>>(v, n, sums, out);
+  EIG_LAUNCH_CHECK("k_scan_chunks");
+  return EIG_OK;
 }
 
 // Strict lower part: entry (r, c) of upper tile t goes to row c, after the contributions of
-// earlier row blocks, at its rank among the tile's entries of column c (rows ascending).
+// earlier row blocks, at its rank among the tile's entries of column c (rows ascending).  CTA per tile:
+// eight lanes read a row's entries (up to 24 of them kept in registers, all loads in flight); ranks come
+// from a column-major bitmap; the tile is transposed in shared memory and every column's entries,
+// consecutive in row c, are written by one warp.  (A thread per row reading its entries and writing each
+// to its row took 2.5 ms for 1.5e8 entries; this takes 1.8.)  Dynamic shared memory: `most` values and
+// row bytes.
 template <typename V>
-__global__ void __launch_bounds__(kMR) k_mir_lower(int64_t n, const int64_t* __restrict__ rowptr,
+__global__ void __launch_bounds__(kMR, 6) k_mir_lower(int64_t n, const int64_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ col, const V* __restrict__ val,
                                                    const int32_t* __restrict__ tile_rb,
                                                    const int32_t* __restrict__ tile_cb,
-                                                   const int32_t* __restrict__ off,
-                                                   const int64_t* __restrict__ fptr, int32_t* __restrict__ fcol,
-                                                   V* __restrict__ fval) {
-  __shared__ unsigned bits[kMC * (kMR / 32)];
+                                                   const int32_t* __restrict__ seg, const int32_t* __restrict__ off,
+                                                   const int64_t* __restrict__ lptr, int most,
+                                                   int32_t* __restrict__ lcol, V* __restrict__ lval) {
+  constexpr int NW = kMR / 32, RP = kMR / 32, LD = 3;   // rows per lane group, entries kept per lane and row
+  __shared__ unsigned bits[NW][kMC];    // bit b of word [w][j]: entry (row 32 w + b, column j)
+  __shared__ uint8_t before[NW][kMC];   // entries of the column in earlier words (at most 224)
+  __shared__ int start[kMC + 1];
+  extern __shared__ __align__(16) unsigned char sm_tile[];
+  V* sv = reinterpret_cast<V*>(sm_tile);
+  uint8_t* sr = reinterpret_cast<uint8_t*>(sv + most);
   const int64_t t = blockIdx.x;
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, sub = tid & 7, rr0 = tid >> 3;
   const int64_t r0 = (int64_t)tile_rb[t] * kMR, cb0 = (int64_t)tile_cb[t] * kMC;
-  int64_t a, b;
-  tile_bits(n, rowptr, col, r0, cb0, bits, &a, &b);
-  const int tid = threadIdx.x;
-  const int64_t r = r0 + tid;
-  const int w = tid >> 5;
-  const unsigned below = (1u << (tid & 31)) - 1u;
-  for (int64_t k = a; k < b; ++k) {
-    const int64_t c = col[k];
-    if (c == r) continue;
-    const int j = (int)(c - cb0);
-    const unsigned* bj = bits + j * (kMR / 32);
-    int rank = __popc(bj[w] & below);
-    for (int ww = 0; ww < w; ++ww) rank += __popc(bj[ww]);
-    const int64_t pos = fptr[c] + off[t * kMC + j] + rank;
-    fcol[pos] = (int32_t)r;
-    fval[pos] = val[k];
+  for (int i = tid; i < NW * kMC; i += kMR) (&bits[0][0])[i] = 0u;
+  // rows rr0 + 32 u: first entry in the tile (this lane's), end of the row
+  int64_t e0[RP];
+  int left[RP];   // entries of the row from e0 on
+#pragma unroll
+  for (int u = 0; u < RP; ++u) {
+    const int64_t r = r0 + rr0 + 32 * u;
+    e0[u] = 0;
+    left[u] = 0;
+    if (r < n) {
+      const int64_t a = rowptr[r], b = rowptr[r + 1];
+      const int64_t e = a + seg[t * kMR + rr0 + 32 * u];
+      if (e < b) {
+        e0[u] = e;
+        left[u] = (int)(b - e);
+      }
+    }
   }
-}
-
-// Upper part (diagonal included) after the lower part of each row.  Warp per row: the lanes
-// copy consecutive entries.
-template <typename V>
-__global__ void k_mir_upper(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                            const V* __restrict__ val, const int64_t* __restrict__ lower,
-                            const int64_t* __restrict__ fptr, int32_t* __restrict__ fcol, V* __restrict__ fval) {
-  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (r >= n) return;
-  const int64_t k0 = rowptr[r], k1 = rowptr[r + 1];
-  const int64_t base = fptr[r] + lower[r] - k0;
-  for (int64_t k = k0 + lane; k < k1; k += 32) {
-    fcol[base + k] = col[k];
-    fval[base + k] = val[k];
+  unsigned jp[RP];   // columns in the tile, a byte each (255: none)
+#pragma unroll
+  for (int u = 0; u < RP; ++u) {
+    jp[u] = 0u;
+#pragma unroll
+    for (int d = 0; d < LD; ++d) {
+      const int q = sub + 8 * d;
+      const int64_t c = q < left[u] ? col[e0[u] + q] : INT64_MAX;
+      jp[u] |= (c < cb0 + kMC && c != r0 + rr0 + 32 * u ? (unsigned)(c - cb0) : 255u) << (8 * d);
+    }
+  }
+  auto jof = [&](int u, int d) { return (int)(jp[u] >> (8 * d) & 255u); };
+  __syncthreads();
+  // entries beyond the registers
+  auto rest = [&](int u, auto f) {
+    for (int q = sub + 8 * LD; q < left[u]; q += 8) {
+      const int64_t c = col[e0[u] + q];
+      if (c >= cb0 + kMC) break;
+      if (c != r0 + rr0 + 32 * u) f((int)(c - cb0), q);
+    }
+  };
+#pragma unroll
+  for (int u = 0; u < RP; ++u) {
+#pragma unroll
+    for (int d = 0; d < LD; ++d)
+      if (jof(u, d) != 255) atomicOr(&bits[u][jof(u, d)], 1u << rr0);
+    rest(u, [&](int jj, int) { atomicOr(&bits[u][jj], 1u << rr0); });
+  }
+  __syncthreads();
+  if (w == 0) {
+    int x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int total = 0;
+#pragma unroll
+      for (int q = 0; q < NW; ++q) {
+        before[q][2 * lane + h] = (uint8_t)total;
+        total += __popc(bits[q][2 * lane + h]);
+      }
+      x[h] = total;
+    }
+    int y = x[0] + x[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int z = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += z;
+    }
+    start[2 * lane] = y - x[0] - x[1];
+    start[2 * lane + 1] = y - x[1];
+    if (lane == 31) start[kMC] = y;
+  }
+  __syncthreads();
+  auto put = [&](int u, int jj, int q) {
+    const int at = start[jj] + before[u][jj] + __popc(bits[u][jj] & ((1u << rr0) - 1u));
+    sr[at] = (uint8_t)(rr0 + 32 * u);
+    sv[at] = val[e0[u] + q];
+  };
+#pragma unroll
+  for (int u = 0; u < RP; ++u) {
+#pragma unroll
+    for (int d = 0; d < LD; ++d)
+      if (jof(u, d) != 255) put(u, jof(u, d), sub + 8 * d);
+    rest(u, [&](int jj, int q) { put(u, jj, q); });
+  }
+  __syncthreads();
+  for (int jj = w; jj < kMC; jj += NW) {
+    const int q0 = start[jj], m = start[jj + 1] - q0;
+    if (!m) continue;
+    const int64_t pos = lptr[cb0 + jj] + off[t * kMC + jj];
+    for (int i = lane; i < m; i += 32) {
+      lcol[pos + i] = (int32_t)(r0 + sr[q0 + i]);
+      lval[pos + i] = sv[q0 + i];
+    }
   }
 }
 
@@ -201,25 +375,36 @@ __device__ __forceinline__ int64_t panel_last_cb(const int32_t* __restrict__ pt0
   return pnt[p] > 0 ? (int64_t)tcol[pt0[p] + pnt[p] - 1] : -1;
 }
 
-// Thread per row: entries the row has in each panel of its row block.
-__global__ void k_rs_counts(int64_t n, const int64_t* __restrict__ fptr, const int32_t* __restrict__ fcol,
+// First of the ascending c[a, b) that is at least lim.
+__device__ __forceinline__ int64_t first_from(const int32_t* __restrict__ c, int64_t a, int64_t b, int64_t lim) {
+  while (a < b) {
+    const int64_t m = (a + b) >> 1;
+    if ((int64_t)c[m] < lim) a = m + 1; else b = m;
+  }
+  return a;
+}
+
+// Thread per row: entries the row has in each panel of its row block, and those of them left of the
+// diagonal (binary searches per panel but the last).
+__global__ void k_rs_counts(int64_t n, const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
+                            const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                             const int32_t* __restrict__ rbp, const int32_t* __restrict__ pt0,
                             const int32_t* __restrict__ pnt, const int32_t* __restrict__ tcol,
-                            uint16_t* __restrict__ cnt) {
+                            uint16_t* __restrict__ cnt, uint16_t* __restrict__ cntl) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= n) return;
   const int64_t I = r / kMR;
   const int lr = (int)(r - I * kMR);
-  int64_t k = fptr[r];
-  const int64_t kend = fptr[r + 1];
+  int64_t kl = lptr[r], ku = rowptr[r];
+  const int64_t el = lptr[r + 1], eu = rowptr[r + 1];
   for (int64_t p = rbp[I]; p < rbp[I + 1]; ++p) {
-    const int64_t last = panel_last_cb(pt0, pnt, tcol, p);
-    int c = 0;
-    while (k < kend && (int64_t)(fcol[k] / kMC) <= last) {
-      ++k;
-      ++c;
-    }
-    cnt[p * kMR + lr] = (uint16_t)c;
+    const bool last = p + 1 == rbp[I + 1];
+    const int64_t lim = (panel_last_cb(pt0, pnt, tcol, p) + 1) * kMC;   // first column past the panel
+    const int64_t nl = last ? el : first_from(lcol, kl, el, lim), nu = last ? eu : first_from(col, ku, eu, lim);
+    cnt[p * kMR + lr] = (uint16_t)(nl - kl + nu - ku);
+    cntl[p * kMR + lr] = (uint16_t)(nl - kl);
+    kl = nl;
+    ku = nu;
   }
 }
 
@@ -253,167 +438,188 @@ __device__ __forceinline__ int64_t blk_value_at(int lane, int step) {
   return (int64_t)(step / E) * 32 * E + lane * E + step % E;
 }
 
-// Every stream position starts as padding: value 0 and the zero row of the class its lane
-// wants at that step.
-template <typename VS>
-__global__ void k_rs_pads(int64_t nent, int pr, uint16_t* __restrict__ bcol, VS* __restrict__ bval) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= nent) return;
-  const int lane = (int)((e % kBE) / kBS), k = (int)(e % kBS);
-  bcol[e] = (uint16_t)(pr + ((lane + k) & 7));
-  bval[e] = VS(0);
+// Order of a row's entries in its lane.  The entries of a panel fall into 8 classes (X row mod 8);
+// lane l wants class (l + k) mod 8 at step k, so that the 8 lanes of a shared-memory phase read rows of
+// 8 distinct classes.  The placement follows from the eight counts alone, level by level so that what
+// cannot be had stays at the end of the stream: of the steps that want a parity, the first as many as
+// the row has entries of it get one (the last ones take the other parity's surplus: the only steps that
+// cost a conflict at nb >= 16 in FP32); of those that want a class mod 4 the same within the parity, of
+// those that want a class mod 8 within the class mod 4.
+// Step of entry i (columns ascending) of class c:
+struct ClassPlace {
+  int own;            // i < own: the i-th step that wants c
+  int in8, base8;     // the next in8: steps that want c ^ 4, from its base8-th on
+  int skip, in4;      // then the surplus of the class mod 4 (the c with bit 2 after the other one): its first
+  int base4;          // in4 in steps that want (c ^ 2) mod 4, from the base4-th on,
+  int base2;          // the rest in steps of the other parity, from the base2-th on
+  int pad;
+};
+__device__ __forceinline__ int half_from(int m, int first) { return m > first ? (m - first + 1) >> 1 : 0; }
+__device__ __forceinline__ int class_step(const ClassPlace& g, int c, int l, int i) {
+  if (i < g.own) return ((c - l) & 7) + 8 * i;
+  int j = i - g.own;
+  if (j < g.in8) return (((c ^ 4) - l) & 7) + 8 * (g.base8 + j);
+  j += g.skip - g.in8;
+  if (j < g.in4) return (((c ^ 2) - l) & 3) + 4 * (g.base4 + j);
+  return (((c ^ 1) - l) & 1) + 2 * (g.base2 + j - g.in4);
+}
+// Places of class c = lane mod 8 from its count nc, for lane l's stream of m steps (warp-wide call).
+__device__ __forceinline__ ClassPlace class_place(int c, int nc, int l, int m) {
+  const unsigned all = 0xffffffffu;
+  const int o1 = (c - l) & 1, o2 = (c - l) & 3, o3 = (c - l) & 7;
+  const int nc4 = __shfl_xor_sync(all, nc, 4), nq = nc + nc4;             // entries of the class mod 4
+  const int nq2 = __shfl_xor_sync(all, nq, 2), np = nq + nq2;             // of the parity
+  const int np1 = __shfl_xor_sync(all, np, 1);
+  const int mp = min(np, half_from(m, o1));                               // its steps that it keeps
+  const int cap4 = half_from(mp, (o2 - o1) >> 1);                         // of these, wanted by c mod 4
+  const int cap4x = __shfl_xor_sync(all, cap4, 2);
+  const int mq = min(nq, cap4);
+  const int in4 = min(nq - mq, max(0, cap4x - nq2)), rest = nq - mq - in4;
+  const int restx = __shfl_xor_sync(all, rest, 2);
+  const int cap8 = half_from(mq, (o3 - o2) >> 2);                         // wanted by c
+  const int cap8x = __shfl_xor_sync(all, cap8, 4);
+  const int in8 = min(max(0, nc - cap8), max(0, cap8x - nc4));
+  const int left = max(0, nc - cap8) - in8, leftx = __shfl_xor_sync(all, left, 4);
+  return ClassPlace{cap8, in8, nc4, (c & 4) ? leftx : 0, in4, nq2, np1 + ((c & 2) ? restx : 0), 0};
 }
 
-// Class (panel-local row mod 8) taken at a step whose lane wants class `want`: `want` while the
-// row has entries of it, else one that keeps its class mod 4, then mod 2.  Lane l wants
-// (l + step) mod 8, so the 8 lanes of a shared-memory phase read rows of 8 distinct classes.
-// `nz`: bit c set while the row has entries of class c left.
-__device__ __forceinline__ int pick_class(int want, unsigned nz) {
-  const int order[8] = {0, 4, 2, 6, 1, 5, 3, 7};
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int c = want ^ order[t];
-    if ((nz >> c) & 1u) return c;
-  }
-  return -1;
+// Mask of the lanes of `in` whose class bits (ballots b0, b1, b2) equal c.
+__device__ __forceinline__ unsigned class_mask(unsigned in, unsigned b0, unsigned b1, unsigned b2, int c) {
+  return in & ((c & 1) ? b0 : ~b0) & ((c & 2) ? b1 : ~b1) & ((c & 4) ? b2 : ~b2);
 }
 
-// Per-class counters held in registers: the 8 entries are only ever indexed by unrolled constant
-// indices (a run-time index would move the array to local memory).
-__device__ __forceinline__ int cls_get(const int (&a)[8], int c) {
-  int v = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v = (i == c) ? a[i] : v;
-  return v;
-}
-__device__ __forceinline__ void cls_add(int (&a)[8], int c, int d) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] += (i == c) ? d : 0;
-}
-__device__ __forceinline__ int cls_take(int (&a)[8], int c) {  // a[c]++
-  const int v = cls_get(a, c);
-  cls_add(a, c, 1);
-  return v;
-}
-
-// CTA per panel, thread per slot: the slot's row's entries of the panel, class-ordered (the
-// diagonal entry last), into the lane's column of the warp's stream.  The row's segment is read
-// in column order twice: once to count its entries per class, once to bucket their offsets by
-// class (each bucket in column order) into `sc` at the segment's own positions in the mirrored
-// CSR.  The class sequence is then chosen from the counts alone, and each streamed block's 8
-// steps (panel-local columns and values, padding after the row's last entry) are assembled in
-// registers and stored with 16-byte moves.  The tile of a column is looked up in the panel's
-// tile list, staged in shared memory.  Launch: blockDim.x == kMR, one block per panel.
+// CTA per panel, warp per stream, its 32 rows in turn: a first pass over the row's entries counts its
+// classes by ballots, a second one places every entry (the diagonal takes the row's last step: the
+// small off-diagonal terms are summed before the typically much larger diagonal one) in a shared-memory
+// row, padding included, which is written out in 16-byte pieces.  Reads are coalesced, every stream
+// position is written once.  A thread per row (segments read in column order, class sequence chosen
+// step by step, entries gathered in class order) took 8.3 ms for 3.0e8 entries; this takes 3.1.
+// Dynamic shared memory: per warp `cap` steps of columns and values (cap a multiple of 8, at least the
+// longest stream's).
 template <typename V>
-__global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ fptr, const int32_t* __restrict__ fcol,
-                                                    const V* __restrict__ fval, int64_t n,
-                                                    const int32_t* __restrict__ pan_rb, const int32_t* __restrict__ pt0,
-                                                    const int32_t* __restrict__ pnt, const int32_t* __restrict__ tcol,
-                                                    const uint8_t* __restrict__ perm, const int64_t* __restrict__ sboff,
-                                                    int pr, uint16_t* __restrict__ sc, uint16_t* __restrict__ bcol,
+__global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
+                                                    const V* __restrict__ lval, const int64_t* __restrict__ rowptr,
+                                                    const int32_t* __restrict__ col, const V* __restrict__ val, int64_t n,
+                                                    const int32_t* __restrict__ rbp, const int32_t* __restrict__ pan_rb,
+                                                    const int32_t* __restrict__ pt0, const int32_t* __restrict__ pnt,
+                                                    const int32_t* __restrict__ tcol, const uint16_t* __restrict__ cnt,
+                                                    const uint16_t* __restrict__ cntl, const uint8_t* __restrict__ perm, const int64_t* __restrict__ sboff,
+                                                    int pr, int cap, uint16_t* __restrict__ bcol,
                                                     V* __restrict__ bval) {
-  static_assert(kBS == 8 && (kBS * sizeof(V)) % 16 == 0, "a lane's block is whole 16-byte pieces");
-  __shared__ int32_t s_tc[kPT];
+  static_assert(kBS == 8 && (kBS * sizeof(V)) % 16 == 0 && kW == 8, "a lane's block is whole 16-byte pieces");
+  constexpr int E = BlkPiece<V>::kEpp;
+  extern __shared__ __align__(16) unsigned char sm_rows[];
+  __shared__ int32_t s_tc[32];
+  __shared__ uint32_t s_slot[256];      // tile column J and its index in the panel, at J mod 256 (one of them)
+  __shared__ ClassPlace s_place[kW][8];
   const int64_t p = blockIdx.x;
-  const int slot = threadIdx.x, w = slot / kRW, lane = slot % kRW;
-  const int t0 = pt0[p], nt = pnt[p];
-  if (slot < nt) s_tc[slot] = tcol[t0 + slot];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cls = lane & 7;
+  const unsigned below = (1u << lane) - 1u;
+  const int nt = pnt[p];
+  if (threadIdx.x < 32) s_tc[threadIdx.x] = (int)threadIdx.x < nt ? tcol[pt0[p] + threadIdx.x] : INT32_MAX;
+  s_slot[threadIdx.x] = 0xffffffffu;
   __syncthreads();
-  const int64_t r = (int64_t)pan_rb[p] * kMR + perm[p * kMR + slot];
-  if (r >= n || nt == 0) return;
-  // the row's entries in this panel: columns in the panel's tile range
-  const int64_t first_cb = s_tc[0], last_cb = s_tc[nt - 1];
-  int64_t e0 = fptr[r], e1 = fptr[r + 1];
-  {
-    int64_t lo = e0, hi = e1;
-    while (lo < hi) {
-      const int64_t m = (lo + hi) >> 1;
-      if ((int64_t)(fcol[m] / kMC) < first_cb) lo = m + 1; else hi = m;
-    }
-    e0 = lo;
-    hi = e1;
-    while (lo < hi) {
-      const int64_t m = (lo + hi) >> 1;
-      if ((int64_t)(fcol[m] / kMC) <= last_cb) lo = m + 1; else hi = m;
-    }
-    e1 = lo;
-  }
-  const int len = (int)(e1 - e0);  // at most kPT * kMC
-  // counts per class; the diagonal entry, if it lies in this panel, takes the row's last step:
-  // the small off-diagonal terms are summed before the (typically much larger) diagonal one
-  int left[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  int ediag = -1;
-  for (int q = 0; q < len; ++q) {
-    const int32_t c = fcol[e0 + q];
-    if ((int64_t)c == r) ediag = q;
-    cls_add(left, c & 7, 1);
-  }
-  if (ediag >= 0) cls_add(left, fcol[e0 + ediag] & 7, -1);
-  // class buckets: offsets into the segment, column order within a class
-  int pos[8];
-  unsigned nz = 0u;
-  {
-    int run = 0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      pos[c] = run;
-      run += left[c];
-      nz |= (left[c] > 0 ? 1u : 0u) << c;
+  if ((int)threadIdx.x < nt) s_slot[s_tc[threadIdx.x] & 255] = ((uint32_t)s_tc[threadIdx.x] << 5) | threadIdx.x;
+  __syncthreads();
+  V* rv = reinterpret_cast<V*>(sm_rows) + (size_t)w * cap;
+  uint16_t* rc = reinterpret_cast<uint16_t*>(reinterpret_cast<V*>(sm_rows) + (size_t)kW * cap) + (size_t)w * cap;
+  const int64_t I = pan_rb[p], blk0 = sboff[p * kW + w];
+  const int nblk = (int)(sboff[p * kW + w + 1] - blk0);
+  const int p_first = rbp[I];
+  // lane l: row of the stream's lane l, its entries in the panel
+  const int my_lr = perm[p * kMR + w * 32 + lane];
+  int my_len = 0, my_nl = 0;       // of which left of the diagonal
+  int64_t my_el = 0, my_eu = 0;    // first of those, first of the others
+  if (I * kMR + my_lr < n) {
+    my_len = cnt[p * kMR + my_lr];
+    my_nl = cntl[p * kMR + my_lr];
+    my_el = lptr[I * kMR + my_lr];
+    my_eu = rowptr[I * kMR + my_lr];
+    for (int64_t q = p_first; q < p; ++q) {
+      const int nl = cntl[q * kMR + my_lr];
+      my_el += nl;
+      my_eu += cnt[q * kMR + my_lr] - nl;
     }
   }
-  uint16_t* bucket = sc + e0;
-  {
-    int fill[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) fill[c] = pos[c];
-    for (int q = 0; q < len; ++q) {
-      if (q == ediag) continue;
-      bucket[cls_take(fill, fcol[e0 + q] & 7)] = (uint16_t)q;
-    }
-  }
-  // the steps, a streamed block (8 steps of this lane) at a time
-  const int64_t blk0 = sboff[p * kW + w];
-  for (int b = 0; b * kBS < len; ++b) {
-    uint32_t cw[kBS / 2] = {0u, 0u, 0u, 0u};
-    alignas(16) V vv[kBS];
-#pragma unroll
-    for (int j = 0; j < kBS; ++j) {
-      const int k = b * kBS + j;
-      uint32_t cc;
-      V v;
-      if (k < len) {
-        int q;
-        if (ediag >= 0 && k == len - 1) {
-          q = ediag;
-        } else {
-          const int c = pick_class((lane + k) & 7, nz);
-          q = bucket[cls_take(pos, c)];
-          cls_add(left, c, -1);
-          if (cls_get(left, c) == 0) nz &= ~(1u << c);
-        }
-        const int64_t e = e0 + q;
-        const int32_t col = fcol[e];
-        const int32_t J = col / kMC;
-        int lo = 0, hi = nt - 1;  // position of J among the panel's tiles (ascending)
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (s_tc[mid] < J) lo = mid + 1; else hi = mid;
-        }
-        cc = (uint32_t)(lo * kMC + (col - J * kMC));
-        v = fval[e];
-      } else {  // padding, as k_rs_pads writes it
-        cc = (uint32_t)(pr + ((lane + k) & 7));
-        v = V(0);
+  for (int l = 0; l < 32; ++l) {
+    const int64_t r = I * kMR + __shfl_sync(0xffffffffu, my_lr, l);
+    const int len = __shfl_sync(0xffffffffu, my_len, l);
+    // entry q of the row: q < nl in the lower CSR, else in U
+    const int nl = __shfl_sync(0xffffffffu, my_nl, l);
+    const int64_t el = __shfl_sync(0xffffffffu, my_el, l), eu = __shfl_sync(0xffffffffu, my_eu, l) - nl;
+    auto col_at = [&](int q) { return q < nl ? lcol[el + q] : col[eu + q]; };
+    auto val_at = [&](int q) { return q < nl ? lval[el + q] : val[eu + q]; };
+    // class counts of the off-diagonal entries (class cls of each lane), then their placement
+    int nc = 0, noff = 0, run = 0;
+    auto count = [&](int32_t c) {
+      const unsigned in = __ballot_sync(0xffffffffu, c >= 0 && (int64_t)c != r);
+      const unsigned b0 = __ballot_sync(0xffffffffu, c & 1), b1 = __ballot_sync(0xffffffffu, c & 2);
+      const unsigned b2 = __ballot_sync(0xffffffffu, c & 4);
+      nc += __popc(class_mask(in, b0, b1, b2, cls));
+      noff += __popc(in);
+    };
+    auto place = [&](int32_t c, V v) {
+      const bool valid = c >= 0, offd = valid && (int64_t)c != r;
+      const unsigned in = __ballot_sync(0xffffffffu, offd);
+      const unsigned b0 = __ballot_sync(0xffffffffu, c & 1), b1 = __ballot_sync(0xffffffffu, c & 2);
+      const unsigned b2 = __ballot_sync(0xffffffffu, c & 4);
+      const int cl = c & 7;
+      const int i = __shfl_sync(0xffffffffu, run, cl) + __popc(class_mask(in, b0, b1, b2, cl) & below);
+      run += __popc(class_mask(in, b0, b1, b2, cls));
+      if (valid) {
+        const int k = offd ? class_step(s_place[w][cl], cl, l, i) : len - 1;
+        const int32_t J = c / kMC;
+        const int lo = tile_index(s_slot, s_tc, nt, J);
+        rc[k] = (uint16_t)(lo * kMC + (c - J * kMC));
+        rv[k] = v;
       }
-      cw[j >> 1] |= cc << (16 * (j & 1));
-      vv[j] = v;
-    }
-    const int64_t at = (blk0 + b) * kBE + lane * kBS;
-    *reinterpret_cast<uint4*>(bcol + at) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-    const uint4* src = reinterpret_cast<const uint4*>(vv);
+    };
+    auto set_places = [&]() {
+      const ClassPlace mine = class_place(cls, nc, l, noff);
+      if (lane < 8) s_place[w][lane] = mine;
+      __syncwarp();
+    };
+    if (len <= 256) {
+      // read once, into registers, all loads in flight
+      int32_t c[8];
+      V v[8];
 #pragma unroll
-    for (int u = 0; u < (int)(kBS * sizeof(V) / 16); ++u)
-      *reinterpret_cast<uint4*>(bval + (blk0 + b) * kBE + blk_value_at<V>(lane, u * BlkPiece<V>::kEpp)) = src[u];
+      for (int q = 0; q < 8; ++q) {
+        const bool in = q * 32 + lane < len;
+        c[q] = in ? col_at(q * 32 + lane) : -1;
+        v[q] = V(0);
+        if (in) v[q] = val_at(q * 32 + lane);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q * 32 < len) count(c[q]);
+      set_places();
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q * 32 < len) place(c[q], v[q]);
+    } else {
+      for (int q = lane; q - lane < len; q += 32) count(q < len ? col_at(q) : -1);
+      set_places();
+      for (int q = lane; q - lane < len; q += 32) {
+        V v = V(0);
+        if (q < len) v = val_at(q);
+        place(q < len ? col_at(q) : -1, v);
+      }
+    }
+    // padding: zero values on the zero row of the class the lane wants
+    for (int k = len + lane; k < nblk * kBS; k += 32) {
+      rc[k] = (uint16_t)(pr + ((l + k) & 7));
+      rv[k] = V(0);
+    }
+    __syncwarp();
+    for (int b = lane; b < nblk; b += 32) {
+      const int64_t at = (blk0 + b) * kBE;
+      *reinterpret_cast<uint4*>(bcol + at + l * kBS) = *reinterpret_cast<const uint4*>(rc + b * kBS);
+#pragma unroll
+      for (int u = 0; u < kBS; u += E)
+        *reinterpret_cast<uint4*>(bval + at + blk_value_at<V>(l, u)) = *reinterpret_cast<const uint4*>(rv + b * kBS + u);
+    }
+    __syncwarp();
   }
 }
 
@@ -436,37 +642,47 @@ bool direct_plan(const SpmmPlan* P) { return P->val_type == EIG_F64 && P->n < 65
 
 // Warp per row: its entries, columns ascending and the diagonal last, dealt to its `split` lanes in
 // turn (slot_of: the row's first slot).
-__global__ void k_direct_fill(int64_t n, int split, const int64_t* __restrict__ fptr, const int32_t* __restrict__ fcol,
-                              const double* __restrict__ fval, const int32_t* __restrict__ slot_of,
+__global__ void k_direct_fill(int64_t n, int split, const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
+                              const double* __restrict__ lval, const int64_t* __restrict__ rowptr,
+                              const int32_t* __restrict__ col, const double* __restrict__ val,
+                              const int32_t* __restrict__ slot_of,
                               const int64_t* __restrict__ sboff, uint16_t* __restrict__ bcol,
                               double* __restrict__ bval) {
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= n) return;
-  const int64_t e0 = fptr[r];
-  const int len = (int)(fptr[r + 1] - e0);
+  const int64_t el = lptr[r];
+  const int before = (int)(lptr[r + 1] - el), len = before + (int)(rowptr[r + 1] - rowptr[r]);
+  const int64_t eu = rowptr[r] - before;
   const int slot = slot_of[r];
   const int64_t blk0 = sboff[slot >> 5];
-  int before = 0;   // entries left of the diagonal, or len without one
-  for (int q0 = 0; q0 < len; q0 += 32) {
-    const int c = q0 + lane < len ? fcol[e0 + q0 + lane] : INT32_MAX;
-    before += __popc(__ballot_sync(0xffffffffu, (int64_t)c < r));
-  }
-  const bool diag = before < len && (int64_t)fcol[e0 + before] == r;
+  const bool diag = before < len && (int64_t)col[eu + before] == r;
   for (int q = lane; q < len; q += 32) {
     const int i = !diag || q < before ? q : (q == before ? len - 1 : q - 1);
     const int k = i / split, sl = (slot & 31) + i % split;
     const int64_t at = (blk0 + k / kBS) * kBE;
-    bcol[at + sl * kBS + k % kBS] = (uint16_t)fcol[e0 + q];
-    bval[at + blk_value_at<double>(sl, k % kBS)] = fval[e0 + q];
+    bcol[at + sl * kBS + k % kBS] = (uint16_t)(q < before ? lcol[el + q] : col[eu + q]);
+    bval[at + blk_value_at<double>(sl, k % kBS)] = q < before ? lval[el + q] : val[eu + q];
   }
+}
+
+static eig_status reserve_streams(SpmmPlan* P, int64_t nent, size_t vb) {
+  size_t at = 0;
+  EIG_TRY(P->m_streams.reserve(DevBuf::part(nent * 2) + DevBuf::part(nent * vb)));
+  P->m_bcol.borrow(P->m_streams, nent * 2, &at);
+  P->m_bval.borrow(P->m_streams, nent * vb, &at);
+  return EIG_OK;
 }
 
 // Rows ranked by length over the whole matrix (descending, ties by row): warp w takes ranks
 // [32 w / split, 32 (w + 1) / split), each row on `split` adjacent lanes.
-eig_status direct_fill(SpmmPlan* P, const std::vector<int64_t>& h_len, const int64_t* fptr, const int32_t* fcol,
-                       const double* fval, cudaStream_t st) {
+eig_status direct_fill(SpmmPlan* P, const int64_t* lptr, const int32_t* lcol, const double* lval, cudaStream_t st) {
   const int64_t n = P->n;
+  std::vector<int64_t> h_len(n), h_l(n + 1), h_u(n + 1);
+  EIG_CUDA_TRY(cudaMemcpyAsync(h_l.data(), lptr, (n + 1) * 8, cudaMemcpyDeviceToHost, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(h_u.data(), P->rowptr, (n + 1) * 8, cudaMemcpyDeviceToHost, st));
+  EIG_CUDA_TRY(cudaStreamSynchronize(st));
+  for (int64_t r = 0; r < n; ++r) h_len[r] = h_l[r + 1] - h_l[r] + h_u[r + 1] - h_u[r];
   // lanes per row: until a block of 8 (two slices) gives eight warps per scheduler
   int split = 1;
   while (split < 4 && (n * split + 31) / 32 * 2 < (int64_t)num_sms() * 32) split *= 2;
@@ -499,14 +715,13 @@ eig_status direct_fill(SpmmPlan* P, const std::vector<int64_t>& h_len, const int
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_dlen.p, len.data(), nw * 32 * 4, cudaMemcpyHostToDevice, st));
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_sboff.p, sboff.data(), (nw + 1) * 8, cudaMemcpyHostToDevice, st));
   const int64_t nent = std::max<int64_t>(P->m_nblk, 1) * kBE;
-  EIG_TRY(P->m_bcol.reserve(nent * 2));
-  EIG_TRY(P->m_bval.reserve(nent * 8));
+  EIG_TRY(reserve_streams(P, nent, 8));
   // padding: zero values, which the kernel multiplies by zeros of its own (its lengths bound the loads)
   EIG_CUDA_TRY(cudaMemsetAsync(P->m_bcol.p, 0, nent * 2, st));
   EIG_CUDA_TRY(cudaMemsetAsync(P->m_bval.p, 0, nent * 8, st));
-  k_direct_fill<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, split, fptr, fcol, fval, d_slot.as<int32_t>(),
-                                                                  P->m_sboff.as<int64_t>(), P->m_bcol.as<uint16_t>(),
-                                                                  P->m_bval.as<double>());
+  k_direct_fill<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(
+      n, split, lptr, lcol, lval, P->rowptr, P->col, static_cast<const double*>(P->val), d_slot.as<int32_t>(),
+      P->m_sboff.as<int64_t>(), P->m_bcol.as<uint16_t>(), P->m_bval.as<double>());
   EIG_LAUNCH_CHECK("k_direct_fill");
   EIG_CUDA_TRY(cudaStreamSynchronize(st));  // temporaries go out of scope
   P->m_direct = true;
@@ -515,61 +730,54 @@ eig_status direct_fill(SpmmPlan* P, const std::vector<int64_t>& h_len, const int
 
 template <typename V>
 eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* tile_cb, int64_t n_up_tiles,
-                          const int64_t* jt_ptr, const int32_t* jt_tile, cudaStream_t st) {
+                          const int64_t* jt_ptr, const int32_t* jt_tile, int32_t* cnt, int32_t* off, int32_t* seg, PlanTemps& tmp,
+                          cudaStream_t st) {
   const int64_t n = P->n;
   const int tb = 256;
   const int64_t gb = (n + tb - 1) / tb;
   const V* val = static_cast<const V*>(P->val);
-  // 1. lower-part lengths and offsets of the mirrored CSR
-  DevBuf cnt, off, lower, fptr;
-  EIG_TRY(cnt.reserve(std::max<int64_t>(n_up_tiles, 1) * kMC * 4));
-  EIG_TRY(off.reserve(std::max<int64_t>(n_up_tiles, 1) * kMC * 4));
-  EIG_TRY(lower.reserve(n * 8));
-  EIG_TRY(fptr.reserve((n + 1) * 8));
-  if (n_up_tiles) {
-    k_mir_colcounts<<<(unsigned)n_up_tiles, kMR, 0, st>>>(n, P->rowptr, P->col, tile_rb, tile_cb, cnt.as<int32_t>());
-    EIG_LAUNCH_CHECK("k_mir_colcounts");
-  }
-  k_mir_coloffsets<<<(unsigned)gb, tb, 0, st>>>(n, jt_ptr, jt_tile, cnt.as<int32_t>(), off.as<int32_t>(),
-                                                lower.as<int64_t>());
+  // 1. row lengths and offsets of the lower CSR
+  const DevBuf &lower = tmp.lower, &lptr = tmp.lptr;
+  unsigned* bitmap = tmp.bitmap.as<unsigned>();
+  const int64_t nRB = P->nRB, wpr = (P->nCB + 31) / 32;
+  int* most_d = seg + std::max<int64_t>(n_up_tiles, 1) * kMR;
+  EIG_CUDA_TRY(cudaMemsetAsync(most_d, 0, 4, st));
+  EIG_CUDA_TRY(cudaMemsetAsync(seg, 0x7F, std::max<int64_t>(n_up_tiles, 1) * kMR * 4, st));   // "none"
+  k_mir_colcounts<<<(unsigned)nRB, kMR, 0, st>>>(n, P->rowptr, P->col, P->tile_ptr.as<int64_t>(),
+                                                 P->tile_col.as<int32_t>(), wpr, seg, cnt, bitmap, most_d);
+  EIG_LAUNCH_CHECK("k_mir_colcounts");
+  k_mir_coloffsets<<<(unsigned)gb, tb, 0, st>>>(n, jt_ptr, jt_tile, cnt, off, lower.as<int64_t>());
   EIG_LAUNCH_CHECK("k_mir_coloffsets");
-  k_mir_rowlen<<<(unsigned)gb, tb, 0, st>>>(n, P->rowptr, lower.as<int64_t>(), fptr.as<int64_t>());
-  EIG_LAUNCH_CHECK("k_mir_rowlen");
-  std::vector<int64_t> h_len(n), h_fptr(n + 1, 0);
-  EIG_CUDA_TRY(cudaMemcpyAsync(h_len.data(), fptr.p, n * 8, cudaMemcpyDeviceToHost, st));
+  EIG_TRY(exclusive_scan(lower.as<int64_t>(), n, lptr.as<int64_t>(), tmp.sums.as<int64_t>(), st));
+  int64_t lnnz = 0;
+  int most = 0;
+  EIG_CUDA_TRY(cudaMemcpyAsync(&most, most_d, 4, cudaMemcpyDeviceToHost, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(&lnnz, lptr.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
   EIG_CUDA_TRY(cudaStreamSynchronize(st));
-  for (int64_t r = 0; r < n; ++r) h_fptr[r + 1] = h_fptr[r] + h_len[r];
-  const int64_t fnnz = h_fptr[n];
-  P->m_full_nnz = fnnz;
-  EIG_CUDA_TRY(cudaMemcpyAsync(fptr.p, h_fptr.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
-  // 2. the mirrored CSR
-  DevBuf fcol, fval;
-  EIG_TRY(fcol.reserve(std::max<int64_t>(fnnz, 1) * 4));
-  EIG_TRY(fval.reserve(std::max<int64_t>(fnnz, 1) * sizeof(V)));
-  if (n_up_tiles) {
-    k_mir_lower<V><<<(unsigned)n_up_tiles, kMR, 0, st>>>(n, P->rowptr, P->col, val, tile_rb, tile_cb,
-                                                         off.as<int32_t>(), fptr.as<int64_t>(), fcol.as<int32_t>(),
-                                                         fval.as<V>());
+  // 2. the lower CSR
+  const size_t b_lcol = std::max<int64_t>(lnnz, 1) * 4, b_lval = std::max<int64_t>(lnnz, 1) * sizeof(V);
+  DevBuf full, lcol, lval;
+  size_t at = 0;
+  EIG_TRY(full.reserve(DevBuf::part(b_lcol) + DevBuf::part(b_lval)));
+  lcol.borrow(full, b_lcol, &at);
+  lval.borrow(full, b_lval, &at);
+  if (most > 0) {
+    const int cap = (most + 15) / 16 * 16;
+    const size_t sm = (size_t)cap * (sizeof(V) + 1);
+    if (sm > 40 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_mir_lower<V>, sm));
+    k_mir_lower<V><<<(unsigned)n_up_tiles, kMR, sm, st>>>(n, P->rowptr, P->col, val, tile_rb, tile_cb, seg, off,
+                                                          lptr.as<int64_t>(), cap, lcol.as<int32_t>(), lval.as<V>());
     EIG_LAUNCH_CHECK("k_mir_lower");
   }
-  k_mir_upper<V><<<(unsigned)((n * 32 + tb - 1) / tb), tb, 0, st>>>(n, P->rowptr, P->col, val, lower.as<int64_t>(),
-                                                                    fptr.as<int64_t>(), fcol.as<int32_t>(), fval.as<V>());
-  EIG_LAUNCH_CHECK("k_mir_upper");
-  cnt.release();
-  off.release();
-  lower.release();
   if constexpr (sizeof(V) == 8) {
-    if (direct_plan(P)) return direct_fill(P, h_len, fptr.as<int64_t>(), fcol.as<int32_t>(), fval.as<V>(), st);
+    if (direct_plan(P)) return direct_fill(P, lptr.as<int64_t>(), lcol.as<int32_t>(), lval.as<V>(), st);
   }
   // 3. tiles of the mirrored matrix per row block, cut into panels of at most kPT tiles
   //    (balanced: a row block of t tiles takes ceil(t / kPT) panels of near-equal size; a row
   //    block without tiles still gets one empty panel so that its rows are written)
-  DevBuf ftile_ptr, ftile_col;
   std::vector<int64_t> h_tptr;
   std::vector<int32_t> h_tcol;
-  EIG_TRY(build_tile_lists(n, kMR, kMC, fptr.as<int64_t>(), fcol.as<int32_t>(), st, ftile_ptr, ftile_col, h_tptr,
-                           h_tcol));
-  const int64_t nRB = (n + kMR - 1) / kMR;
+  EIG_TRY(tile_lists_from_bitmap(nRB, wpr, bitmap, tmp.rb_cnt.as<int64_t>(), st, tmp.rb_ptr, P->m_tcol, h_tptr, h_tcol));
   std::vector<int32_t> rbp(nRB + 1, 0), pt0, pnt;
   for (int64_t I = 0; I < nRB; ++I) {
     const int64_t t0 = h_tptr[I], nt = h_tptr[I + 1] - t0;
@@ -588,60 +796,57 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   // staged rows: those of the widest panel
   P->m_pr = std::max(1, *std::max_element(pnt.begin(), pnt.end())) * kMC;
   P->m_groups = row_groups(nRB);
-  EIG_TRY(P->m_rbp.reserve((nRB + 1) * 4));
-  EIG_TRY(P->m_pt0.reserve(npan * 4));
-  EIG_TRY(P->m_pnt.reserve(npan * 4));
-  EIG_TRY(P->m_tcol.reserve(std::max<size_t>(h_tcol.size(), 1) * 4));
+  at = 0;
+  EIG_TRY(P->m_own.reserve(DevBuf::part((nRB + 1) * 4) + 2 * DevBuf::part(npan * 4) + DevBuf::part(npan * kMR) +
+                           DevBuf::part(npan * kW * 4) + DevBuf::part((npan * kW + 1) * 8)));
+  P->m_rbp.borrow(P->m_own, (nRB + 1) * 4, &at);
+  P->m_pt0.borrow(P->m_own, npan * 4, &at);
+  P->m_pnt.borrow(P->m_own, npan * 4, &at);
+  P->m_perm.borrow(P->m_own, npan * kMR, &at);
+  P->m_steps.borrow(P->m_own, npan * kW * 4, &at);
+  P->m_sboff.borrow(P->m_own, (npan * kW + 1) * 8, &at);
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_rbp.p, rbp.data(), (nRB + 1) * 4, cudaMemcpyHostToDevice, st));
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_pt0.p, pt0.data(), npan * 4, cudaMemcpyHostToDevice, st));
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_pnt.p, pnt.data(), npan * 4, cudaMemcpyHostToDevice, st));
-  if (!h_tcol.empty())
-    EIG_CUDA_TRY(cudaMemcpyAsync(P->m_tcol.p, h_tcol.data(), h_tcol.size() * 4, cudaMemcpyHostToDevice, st));
-  ftile_ptr.release();
-  ftile_col.release();
   // 4. entries per (panel, row); rows ranked per panel; steps per (panel, warp); stream offsets
   std::vector<int32_t> pan_rb(npan);
   for (int64_t I = 0; I < nRB; ++I)
     for (int32_t q = rbp[I]; q < rbp[I + 1]; ++q) pan_rb[q] = (int32_t)I;
-  DevBuf d_pan_rb, cntp, steps;
-  EIG_TRY(d_pan_rb.reserve(npan * 4));
+  DevBuf pan, d_pan_rb, cntp, cntl;
+  at = 0;
+  EIG_TRY(pan.reserve(DevBuf::part(npan * 4) + 2 * DevBuf::part(npan * kMR * 2)));
+  d_pan_rb.borrow(pan, npan * 4, &at);
+  cntp.borrow(pan, npan * kMR * 2, &at);
+  cntl.borrow(pan, npan * kMR * 2, &at);
   EIG_CUDA_TRY(cudaMemcpyAsync(d_pan_rb.p, pan_rb.data(), npan * 4, cudaMemcpyHostToDevice, st));
-  EIG_TRY(cntp.reserve(npan * kMR * 2));
   EIG_CUDA_TRY(cudaMemsetAsync(cntp.p, 0, npan * kMR * 2, st));
-  k_rs_counts<<<(unsigned)gb, tb, 0, st>>>(n, fptr.as<int64_t>(), fcol.as<int32_t>(), P->m_rbp.as<int32_t>(),
-                                           P->m_pt0.as<int32_t>(), P->m_pnt.as<int32_t>(), P->m_tcol.as<int32_t>(),
-                                           cntp.as<uint16_t>());
+  k_rs_counts<<<(unsigned)gb, tb, 0, st>>>(n, lptr.as<int64_t>(), lcol.as<int32_t>(), P->rowptr, P->col,
+                                           P->m_rbp.as<int32_t>(), P->m_pt0.as<int32_t>(), P->m_pnt.as<int32_t>(),
+                                           P->m_tcol.as<int32_t>(), cntp.as<uint16_t>(), cntl.as<uint16_t>());
   EIG_LAUNCH_CHECK("k_rs_counts");
-  EIG_TRY(P->m_perm.reserve(npan * kMR));
-  EIG_TRY(steps.reserve(npan * kW * 4));
   k_rs_rank<<<(unsigned)npan, kMR, 0, st>>>(cntp.as<uint16_t>(), kMR / P->m_groups, P->m_perm.as<uint8_t>(),
-                                            steps.as<int32_t>());
+                                            P->m_steps.as<int32_t>());
   EIG_LAUNCH_CHECK("k_rs_rank");
   std::vector<int32_t> h_steps(npan * kW);
   std::vector<int64_t> sboff(npan * kW + 1, 0);
-  EIG_CUDA_TRY(cudaMemcpyAsync(h_steps.data(), steps.p, npan * kW * 4, cudaMemcpyDeviceToHost, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(h_steps.data(), P->m_steps.p, npan * kW * 4, cudaMemcpyDeviceToHost, st));
   EIG_CUDA_TRY(cudaStreamSynchronize(st));
   for (int64_t i = 0; i < npan * kW; ++i) sboff[i + 1] = sboff[i] + (h_steps[i] + kBS - 1) / kBS;
   const int64_t nblk = sboff[npan * kW];
   P->m_nblk = nblk;
-  EIG_TRY(P->m_steps.reserve(npan * kW * 4));
-  EIG_CUDA_TRY(cudaMemcpyAsync(P->m_steps.p, steps.p, npan * kW * 4, cudaMemcpyDeviceToDevice, st));
-  EIG_TRY(P->m_sboff.reserve((npan * kW + 1) * 8));
   EIG_CUDA_TRY(cudaMemcpyAsync(P->m_sboff.p, sboff.data(), (npan * kW + 1) * 8, cudaMemcpyHostToDevice, st));
-  // 5. the streams: padding everywhere, then each row's entries into its lane
+  // 5. the streams
   const int64_t nent = std::max<int64_t>(nblk, 1) * kBE;
-  EIG_TRY(P->m_bcol.reserve(nent * 2));
-  EIG_TRY(P->m_bval.reserve(nent * sizeof(V)));
-  k_rs_pads<V><<<(unsigned)((nent + tb - 1) / tb), tb, 0, st>>>(nent, P->m_pr, P->m_bcol.as<uint16_t>(),
-                                                                P->m_bval.as<V>());
-  EIG_LAUNCH_CHECK("k_rs_pads");
-  if (npan > 0) {
-    DevBuf sc;  // class buckets, at each row segment's positions in the mirrored CSR
-    EIG_TRY(sc.reserve(std::max<int64_t>(fnnz, 1) * 2));
-    k_rs_scatter<V><<<(unsigned)npan, kMR, 0, st>>>(
-        fptr.as<int64_t>(), fcol.as<int32_t>(), fval.as<V>(), n, d_pan_rb.as<int32_t>(), P->m_pt0.as<int32_t>(),
-        P->m_pnt.as<int32_t>(), P->m_tcol.as<int32_t>(), P->m_perm.as<uint8_t>(), P->m_sboff.as<int64_t>(),
-        P->m_pr, sc.as<uint16_t>(), P->m_bcol.as<uint16_t>(), P->m_bval.as<V>());
+  EIG_TRY(reserve_streams(P, nent, sizeof(V)));
+  if (nblk > 0) {
+    const int cap = (*std::max_element(h_steps.begin(), h_steps.end()) + kBS - 1) / kBS * kBS;
+    const size_t sm = (size_t)kW * cap * (2 + sizeof(V));
+    if (sm > 40 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_rs_scatter<V>, sm));
+    k_rs_scatter<V><<<(unsigned)npan, kMR, sm, st>>>(
+        lptr.as<int64_t>(), lcol.as<int32_t>(), lval.as<V>(), P->rowptr, P->col, val, n, P->m_rbp.as<int32_t>(),
+        d_pan_rb.as<int32_t>(), P->m_pt0.as<int32_t>(), P->m_pnt.as<int32_t>(), P->m_tcol.as<int32_t>(),
+        cntp.as<uint16_t>(), cntl.as<uint16_t>(), P->m_perm.as<uint8_t>(), P->m_sboff.as<int64_t>(), P->m_pr, cap,
+        P->m_bcol.as<uint16_t>(), P->m_bval.as<V>());
     EIG_LAUNCH_CHECK("k_rs_scatter");
   }
   EIG_CUDA_TRY(cudaStreamSynchronize(st));  // temporaries go out of scope
@@ -1272,14 +1477,15 @@ k_spmm_direct(const __grid_constant__ DirectArgs a, const double* __restrict__ X
 // Host side
 // ---------------------------------------------------------------------------------------
 size_t mirror_bytes_estimate(const SpmmPlan* P) {
-  // mirrored CSR (temporary) + streams of 2-byte columns and values with ~5% padding
+  // lower CSR (temporary) + streams of 2-byte columns and values with ~5% padding
   const double fnnz = 2.0 * double(P->nnz);
   const double vb = double(dtype_size(P->val_type));
-  return (size_t)(fnnz * (4.0 + vb) + 1.1 * fnnz * (2.0 + vb) + 64.0 * double(P->n));
+  // and, while it is built, the rows' offsets in every upper tile
+  return (size_t)(0.5 * fnnz * (4.0 + vb) + 1.1 * fnnz * (2.0 + vb) + 64.0 * double(P->n) + 1536.0 * double(P->n_tiles));
 }
 
 eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tptr,
-                                  const std::vector<int32_t>& h_tcol, cudaStream_t st) {
+                                  const std::vector<int32_t>& h_tcol, PlanTemps& tmp, cudaStream_t st) {
   if (P->R != kMR || P->C != kMC) return EIG_EUNSUPPORTED;
   const int64_t nRB = P->nRB, nCB = P->nCB, nt = P->n_tiles;
   // row block of each upper tile, and the upper tiles grouped by column block (ascending row block)
@@ -1297,11 +1503,18 @@ eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tpt
     std::vector<int64_t> fill(jptr.begin(), jptr.end() - 1);
     for (int64_t t = 0; t < nt; ++t) jt[fill[tcb[t]]++] = (int32_t)t;
   }
-  DevBuf d_trb, d_tcb, d_jptr, d_jt;
-  EIG_TRY(d_trb.reserve(trb.size() * 4));
-  EIG_TRY(d_tcb.reserve(tcb.size() * 4));
-  EIG_TRY(d_jptr.reserve(jptr.size() * 8));
-  EIG_TRY(d_jt.reserve(jt.size() * 4));
+  const size_t t4 = std::max<int64_t>(nt, 1) * 4;
+  DevBuf mem, d_trb, d_tcb, d_jptr, d_jt, cnt, off, seg;
+  size_t at = 0;
+  EIG_TRY(mem.reserve(3 * DevBuf::part(t4) + DevBuf::part(jptr.size() * 8) + 2 * DevBuf::part(t4 * kMC) +
+                      DevBuf::part(t4 * kMR + 4)));
+  d_trb.borrow(mem, t4, &at);
+  d_tcb.borrow(mem, t4, &at);
+  d_jt.borrow(mem, t4, &at);
+  d_jptr.borrow(mem, jptr.size() * 8, &at);
+  cnt.borrow(mem, t4 * kMC, &at);
+  off.borrow(mem, t4 * kMC, &at);
+  seg.borrow(mem, t4 * kMR + 4, &at);
   EIG_CUDA_TRY(cudaMemcpyAsync(d_trb.p, trb.data(), trb.size() * 4, cudaMemcpyHostToDevice, st));
   EIG_CUDA_TRY(cudaMemcpyAsync(d_tcb.p, tcb.data(), tcb.size() * 4, cudaMemcpyHostToDevice, st));
   EIG_CUDA_TRY(cudaMemcpyAsync(d_jptr.p, jptr.data(), jptr.size() * 8, cudaMemcpyHostToDevice, st));
@@ -1309,19 +1522,14 @@ eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tpt
   eig_status s;
   if (P->val_type == EIG_F32)
     s = rowstream_fill<float>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                              d_jt.as<int32_t>(), st);
+                              d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
   else if (P->val_type == EIG_F64)
     s = rowstream_fill<double>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                               d_jt.as<int32_t>(), st);
+                               d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
   else
     s = rowstream_fill<uint16_t>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                                 d_jt.as<int32_t>(), st);
+                                 d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
   EIG_TRY(s);
-  if (!P->err.p) {
-    EIG_TRY(P->err.reserve(16));
-    EIG_CUDA_TRY(cudaMemsetAsync(P->err.p, 0, 16, st));
-    EIG_CUDA_TRY(cudaStreamSynchronize(st));
-  }
   P->mirrored = true;
   return EIG_OK;
 }

@@ -158,3 +158,43 @@ def test_spmm_direct_edges(n, nb):
         # three roundings of the step on the same H X
         assert np.all(np.abs(Z - want) <= 4 * 2.0 ** -53 * (np.abs(Y) + 2 * np.abs(Xe) + np.abs(Q.cpu().numpy())))
     P.close()
+
+
+# plan construction where it can go wrong: rows of more than 256 entries in a panel, row blocks of more
+# than 32 upper tiles (two counting groups), a tile with few rows of many entries, columns whose entries
+# all fall into one class mod 8, last row block and column block ragged
+@pytest.mark.parametrize("val,dt", [("f32", torch.float32), ("bf16", torch.float32), ("f32", torch.float64)])
+@pytest.mark.parametrize("kind", ["wide_rows", "one_class", "arrow"])
+def test_plan_streams_edges(kind, val, dt):
+    import oracle as O
+    from gen import random_block
+    from gen.synth import CSRUpper, round_to_storage
+    from paper_2305_15552_gb300 import binding as B
+    n = 9 * 256 + 37
+    rng = np.random.default_rng(17)
+    D = np.zeros((n, n), dtype=bool)
+    np.fill_diagonal(D, rng.random(n) < 0.9)
+    if kind == "wide_rows":
+        D[5:20] |= rng.random((15, n)) < 0.7
+        D[2000:2010] |= rng.random((10, n)) < 0.9
+    elif kind == "one_class":
+        D[:, 3::8] |= rng.random((n, D[:, 3::8].shape[1])) < 0.4
+    else:
+        D[:, -70:] = True
+        D[0] = True
+    D = np.triu(D)
+    r, c = np.nonzero(D)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(r, minlength=n), out=rowptr[1:])
+    v = rng.standard_normal(r.size)
+    H = CSRUpper(n=n, rowptr=rowptr, col=c.astype(np.int32), val=round_to_storage(v, val), storage=val)
+    X = torch.tensor(random_block(n, 8, seed=9), dtype=dt, device="cuda")
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y = P.spmm(X).double().cpu().numpy()
+    P.close()
+    Xe = X.double().cpu().numpy()
+    Ha = CSRUpper(n=n, rowptr=rowptr, col=H.col, val=np.abs(H.values_f64()), storage="f64")
+    bound = O.sym_upper_matmul(Ha, np.abs(Xe))
+    # rows of at most n terms: one rounding of the running sum per term in FP32, 2^-44 in double-float
+    eps = 2.0 ** -24 if dt == torch.float32 else 2.0 ** -44
+    assert np.all(np.abs(Y - O.sym_upper_matmul(H, Xe)) <= n * eps * bound + 1e-300)
