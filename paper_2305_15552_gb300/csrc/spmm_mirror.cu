@@ -887,6 +887,7 @@ struct RsArgs {
   const int64_t* sboff;
   const uint16_t* bcol;
   const void* bval;
+  float minus_zero;   // -0 (see RsAcc<double, N, true>)
   int pr;        // staged rows of the widest panel; the zero rows follow them
   int* err;
 };
@@ -1000,7 +1001,7 @@ template <int N> struct RsAcc<float, N, false> {
   typedef float OT;
   static constexpr int N2 = (N + 1) / 2;
   float2 y[N2];
-  __device__ __forceinline__ void zero() {
+  __device__ __forceinline__ void zero(float) {
 #pragma unroll
     for (int e = 0; e < N2; ++e) y[e] = make_float2(0.0f, 0.0f);
   }
@@ -1023,7 +1024,7 @@ template <int N> struct RsAcc<double, N, false> {
   typedef double VT;
   typedef double OT;
   double y[N];
-  __device__ __forceinline__ void zero() {
+  __device__ __forceinline__ void zero(float) {
 #pragma unroll
     for (int e = 0; e < N; ++e) y[e] = 0.0;
   }
@@ -1034,46 +1035,50 @@ template <int N> struct RsAcc<double, N, false> {
   __device__ __forceinline__ OT get(int e) const { return y[e]; }
 };
 // Double-float: X staged as (hi, lo) FP32 pairs (8 bytes per element, like FP64); each product
-// v * hi taken exactly (FMA two-product), summed into hi by two-sum, every error term and v * lo
-// into lo: ~2^-44 relative per step, at FP32 instruction rate.  A 16-byte piece holds two
-// elements as (hi_e, hi_e+1, lo_e, lo_e+1), so a step is FP32x2 arithmetic on element pairs;
-// every operation is an explicit round-to-nearest (a subtraction b - a is fma(a, -1, b)), so no
-// contraction can break the two-sum.  A one-element piece (block width 1) holds (hi, lo).
+// v * xh is summed into hi by two-sum, every error term and v * xl into lo: ~2^-44 relative per step, at
+// FP32 instruction rate.  With p = v xh rounded, t = hi + p rounded and b = t - hi, the error of both
+// roundings is (hi - (t - b)) + (v xh - b): the first difference is exact and the second is one fused
+// multiply-add, which takes the product's rounding along (v xh - p need not be formed by itself: nine
+// operations instead of eleven, 2.88 -> 2.60 ms at n = 2M, 400 nonzeros a row, nb = 8).  A 16-byte piece
+// holds two elements as (hi_e, hi_e+1, lo_e, lo_e+1), so a step is FP32x2 arithmetic on element pairs;
+// every operation is an explicit round-to-nearest (a subtraction a - b is fma(b, -1, a)).  A one-element
+// piece (block width 1) holds (hi, lo).  The rounded product is fma(v, xh, nz) with nz = -0 from the
+// kernel's arguments: the compiler contracts a packed multiplication and a following packed addition
+// into one fused operation even where both have explicit roundings (also through a constant -0), and
+// the two-sum would then lose its low word (errors of 1e-10 instead of 2e-15).
 template <int N> struct RsAcc<double, N, true> {
   typedef float VT;
   typedef double OT;
   static constexpr int N2 = (N + 1) / 2;
   float2 hi[N2], lo[N2];
-  __device__ __forceinline__ void zero() {
+  float nz;
+  __device__ __forceinline__ void zero(float minus_zero) {
+    nz = minus_zero;
 #pragma unroll
     for (int e = 0; e < N2; ++e) hi[e] = lo[e] = make_float2(0.0f, 0.0f);
   }
   __device__ __forceinline__ void add(int slot0, float v, const uint32_t* w, int nw) {
     if (nw == 4) {
       const int s = slot0 / 2;
-      const float2 vv = make_float2(v, v), nv = make_float2(-v, -v), m1 = make_float2(-1.0f, -1.0f);
+      const float2 vv = make_float2(v, v), m1 = make_float2(-1.0f, -1.0f);
       const float2 xh = make_float2(__uint_as_float(w[0]), __uint_as_float(w[1]));
       const float2 xl = make_float2(__uint_as_float(w[2]), __uint_as_float(w[3]));
-      const float2 p = __fmul2_rn(vv, xh);
-      const float2 q = __ffma2_rn(nv, xh, p);                          // p - v hi: minus the product's error
-      const float2 t = __fadd2_rn(hi[s], p);
-      const float2 bb = __ffma2_rn(hi[s], m1, t);                      // t - hi
-      const float2 e1 = __ffma2_rn(__ffma2_rn(bb, m1, t), m1, hi[s]);  // hi - (t - bb)
-      const float2 e2 = __ffma2_rn(bb, m1, p);                         // p - bb
-      const float2 err = __fadd2_rn(e1, e2);
+      const float2 t = __fadd2_rn(hi[s], __ffma2_rn(vv, xh, make_float2(nz, nz)));
+      const float2 nb = __ffma2_rn(t, m1, hi[s]);                       // hi - t = -b
+      const float2 e1 = __ffma2_rn(__fadd2_rn(t, nb), m1, hi[s]);       // hi - (t - b)
+      const float2 e2 = __ffma2_rn(vv, xh, nb);                         // v xh - b
       hi[s] = t;
-      lo[s] = __ffma2_rn(vv, xl, __fadd2_rn(lo[s], __ffma2_rn(q, m1, err)));
+      lo[s] = __ffma2_rn(vv, xl, __fadd2_rn(lo[s], __fadd2_rn(e1, e2)));
     } else {
       float& h = (slot0 & 1) ? hi[slot0 / 2].y : hi[slot0 / 2].x;
       float& l = (slot0 & 1) ? lo[slot0 / 2].y : lo[slot0 / 2].x;
       const float xh = __uint_as_float(w[0]), xl = __uint_as_float(w[1]);
-      const float p = __fmul_rn(v, xh);
-      const float pe = __fmaf_rn(v, xh, -p);
-      const float t = __fadd_rn(h, p);
-      const float bb = __fsub_rn(t, h);
-      const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+      const float t = __fadd_rn(h, __fmaf_rn(v, xh, nz));
+      const float nb = __fsub_rn(h, t);
+      const float e1 = __fsub_rn(h, __fadd_rn(t, nb));
+      const float e2 = __fmaf_rn(v, xh, nb);
       h = t;
-      l = __fmaf_rn(v, xl, __fadd_rn(l, __fadd_rn(err, pe)));
+      l = __fmaf_rn(v, xl, __fadd_rn(l, __fadd_rn(e1, e2)));
     }
   }
   __device__ __forceinline__ OT get(int e) const {
@@ -1228,7 +1233,7 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
     const int64_t b0 = a.sboff[(int64_t)p * kW + w];
     const int nb = (L + kBS - 1) / kBS;
     Acc acc;
-    acc.zero();
+    acc.zero(a.minus_zero);
     uint4 bc[PF];
     uint32_t bv[PF][VW];
     auto load_blk = [&](int b, int s) {
@@ -1578,6 +1583,7 @@ static RsArgs rs_args(SpmmPlan* P) {
   a.sboff = P->m_sboff.as<int64_t>();
   a.bcol = P->m_bcol.as<uint16_t>();
   a.bval = P->m_bval.p;
+  a.minus_zero = -0.0f;
   a.pr = P->m_pr;
   a.err = P->err.as<int>();
   return a;
