@@ -17,6 +17,41 @@ cudaError_t ensure_dyn_smem(const void* kern, size_t bytes) {
   if (e == cudaSuccess) cur = bytes;
   return e;
 }
+namespace {
+struct ScratchPools {
+  static constexpr int kDevices = 64;
+  std::mutex mu;
+  cudaMemPool_t pool[kDevices] = {};
+  bool tried[kDevices] = {};
+  ~ScratchPools() {   // at unload; errors of a runtime that is already gone are of no interest
+    for (cudaMemPool_t q : pool)
+      if (q) cudaMemPoolDestroy(q);
+  }
+  cudaMemPool_t get(int dev) {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!tried[dev]) {
+      tried[dev] = true;
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = 32u << 20;
+      if (cudaMemPoolCreate(&pool[dev], &props) != cudaSuccess) pool[dev] = nullptr;
+      else cudaMemPoolSetAttribute(pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+      cudaGetLastError();
+    }
+    return pool[dev];
+  }
+};
+}  // namespace
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  static ScratchPools pools;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t q = dev < ScratchPools::kDevices ? pools.get(dev) : nullptr;
+  return q ? cudaMallocFromPoolAsync(p, bytes, q, st) : cudaMallocAsync(p, bytes, st);
+}
 static std::atomic<long long> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 static thread_local char g_cuda_msg[512] = {0};

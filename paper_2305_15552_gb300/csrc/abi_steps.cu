@@ -14,8 +14,8 @@ struct AsyncScratch {
   cudaStream_t st;
   explicit AsyncScratch(cudaStream_t s) : st(s) {}
   eig_status get(size_t bytes) {
-    cudaError_t e = cudaMallocAsync(&p, bytes, st);
-    if (e != cudaSuccess) { set_cuda_error(e, "cudaMallocAsync", __FILE__, __LINE__); p = nullptr; return EIG_ENOMEM; }
+    cudaError_t e = scratch_alloc(&p, bytes, st);
+    if (e != cudaSuccess) { set_cuda_error(e, "scratch_alloc", __FILE__, __LINE__); p = nullptr; return EIG_ENOMEM; }
     return EIG_OK;
   }
   ~AsyncScratch() { if (p) cudaFreeAsync(p, st); }

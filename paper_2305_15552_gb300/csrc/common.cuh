@@ -34,6 +34,11 @@ inline cudaError_t ensure_dyn_smem(K* kern, size_t bytes) {
   return ensure_dyn_smem(reinterpret_cast<const void*>(kern), bytes);
 }
 
+// Stream-ordered scratch of one call, from a pool of the library's own on each device that keeps at
+// most 32 MiB between calls (cudaFreeAsync returns it).  The device's default pool gives its memory back
+// at every synchronisation, after which an allocation maps it anew (0.1 to 0.2 ms).
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
+
 // Count of kernel launches made by this library (every launch site checks through here).
 void count_launch();
 
