@@ -119,6 +119,9 @@ __device__ __forceinline__ dfl scale2(dfl a, int e) {
   const float f = pow2f(e);
   return dfl(a.hi * f, a.lo * f);
 }
+// a * f, exact for f a power of two (the result neither over- nor underflows)
+__device__ __forceinline__ dfl scale_by(dfl a, float f) { return dfl(a.hi * f, a.lo * f); }
+__device__ __forceinline__ double scale_by(double a, float f) { return a * (double)f; }
 __device__ __forceinline__ double scale2(double a, int e) { return a * (double)pow2f(e); }
 
 __device__ __forceinline__ dfl shfl_xor(dfl v, int o) {

@@ -228,9 +228,16 @@ __device__ __forceinline__ int sturm_count(const R* __restrict__ d, const R* __r
   R pm = 1.0, pc = d[0] - x;
   if (lead_f32(pc) == 0.0f) pc = R(-0x1p-40);
   int c = sign_bit(pc);
+  // What bounds it: the recurrence's dependent operations.  The next step's shifted diagonal and e2 are loaded and formed ahead of it, and the rescale is a
+  // multiplication by 1 or 2^+-64 instead of branches (a step at two warps per scheduler: 203 -> 160 cycles;
+  // four warps issue ~68 instructions each and take 255, 273 before).
+  R dn = (k > 1) ? d[1] - x : R(0.0), en = (k > 1) ? e2[0] : R(0.0);
   for (int i = 1; i < k; ++i) {
-    const R t = e2[i - 1] * pm;
-    const R pn = dfma(d[i] - x, pc, -t);
+    const R dx = dn, t = en * pm;
+    const int i1 = min(i + 1, k - 1);
+    dn = d[i1] - x;
+    en = e2[i1 - 1];
+    const R pn = dfma(dx, pc, -t);
     pm = pc;
     pc = (lead_f32(pn) == 0.0f) ? -scale2(pm, -40) : pn;
     c += sign_bit(pc) ^ sign_bit(pm);
@@ -238,8 +245,9 @@ __device__ __forceinline__ int sturm_count(const R* __restrict__ d, const R* __r
     // pair is kept in [2^-64, 2^64]; a minor that still underflows is a pivot below ~2^-62 of
     // the norm, counted as zero (the count of a matrix perturbed that little)
     const float big = fmaxf(fabsf(lead_f32(pc)), fabsf(lead_f32(pm)));
-    if (big > 0x1p64f) { pc = scale2(pc, -64); pm = scale2(pm, -64); }
-    else if (big < 0x1p-64f) { pc = scale2(pc, 64); pm = scale2(pm, 64); }
+    const float f = big > 0x1p64f ? 0x1p-64f : (big < 0x1p-64f ? 0x1p64f : 1.0f);
+    pc = scale_by(pc, f);
+    pm = scale_by(pm, f);
   }
   return c;
 }
@@ -264,50 +272,62 @@ __device__ __forceinline__ void tri_shift_factor(const R* __restrict__ d, const 
     const R sub = e[i];
     const R nd = d[i + 1] - sigma;
     const R ne = (i + 2 < k) ? e[i + 1] : R(0.0);
-    if (fabs(c0) >= fabs(sub)) {
-      const R rc = R(1.0) / guard_tiny(c0, tiny);
-      const R l = sub * rc;
-      u0[i * s] = rc; u1[i * s] = c1; u2[i * s] = R(0.0);
-      lm[i * s] = l;
-      piv[i * s] = 0;
-      c0 = dfma(-l, c1, nd);
-      c1 = ne;
-    } else {
-      const R rs = R(1.0) / guard_tiny(sub, tiny);
-      const R l = c0 * rs;
-      u0[i * s] = rs; u1[i * s] = nd; u2[i * s] = ne;
-      lm[i * s] = l;
-      piv[i * s] = 1;
-      const R t = c1;
-      c0 = dfma(-l, nd, t);
-      c1 = -l * ne;
-    }
+    // selects instead of a branch: a warp's vectors swap rows at different steps, and a branch
+    // would run the division on both sides
+    const bool swap = !(fabs(c0) >= fabs(sub));
+    const R rc = R(1.0) / guard_tiny(swap ? sub : c0, tiny);
+    const R l = (swap ? c0 : sub) * rc;
+    const R up = swap ? nd : c1, dn = swap ? c1 : nd;   // the pivot row's next entry, the other row's
+    u0[i * s] = rc;
+    u1[i * s] = up;
+    u2[i * s] = swap ? ne : R(0.0);
+    lm[i * s] = l;
+    piv[i * s] = swap;
+    c0 = dfma(-l, up, dn);
+    c1 = swap ? -l * ne : ne;
   }
   u0[(k - 1) * s] = R(1.0) / guard_tiny(c0, tiny);
 }
 
-// y <- (T - sigma I)^{-1} y from the factors of tri_shift_factor.
+// y <- (T - sigma I)^{-1} (sc y) from the factors of tri_shift_factor; returns max |y_i|.
 template <typename R>
-__device__ __forceinline__ void tri_shift_apply(int k, const R* __restrict__ u0, const R* __restrict__ u1,
+__device__ __forceinline__ R tri_shift_apply(int k, const R* __restrict__ u0, const R* __restrict__ u1,
                                                 const R* __restrict__ u2, const R* __restrict__ lm,
-                                                const unsigned char* __restrict__ piv, int s, R* __restrict__ y) {
-  R yc = y[0];
+                                                const unsigned char* __restrict__ piv, int s, R* __restrict__ y, R sc) {
+  // each step's operands are loaded a step ahead of the recurrence
+  const int kl = k - 2;                  // last factor entry of the forward pass
+  R yc = y[0] * sc;
+  R yl = (k > 1) ? y[1] * sc : R(0.0), ll = (k > 1) ? lm[0] : R(0.0);
+  bool sw = k > 1 && piv[0];
   for (int i = 0; i + 1 < k; ++i) {
-    R yn = y[i + 1];
-    if (piv[i * s]) { const R t = yc; yc = yn; yn = t; }
-    y[i] = yc;
-    yc = dfma(-lm[i * s], yc, yn);
+    const R yn = sw ? yc : yl, yi = sw ? yl : yc, l = ll;
+    const int i1 = min(i + 1, kl);
+    yl = y[i1 + 1] * sc;
+    ll = lm[i1 * s];
+    sw = piv[i1 * s];
+    y[i] = yi;
+    yc = dfma(-l, yi, yn);
   }
   R y1 = yc * u0[(k - 1) * s];           // y[i+1]
   y[k - 1] = y1;
+  R ymx = fmax(R(0.0), fabs(y1));
   R y2 = 0.0;                            // y[i+2]
-  for (int i = k - 2; i >= 0; --i) {
-    const R t = dfma(-u2[i * s], y2, y[i]);
-    const R yi = dfma(-u1[i * s], y1, t) * u0[i * s];
+  const int k2 = max(kl, 0);
+  R yv = y[k2], v0 = u0[k2 * s], v1 = (k > 1) ? u1[k2 * s] : R(0.0), v2 = (k > 1) ? u2[k2 * s] : R(0.0);
+  for (int i = kl; i >= 0; --i) {
+    const R t = dfma(-v2, y2, yv), w1 = -v1, w0 = v0;
+    const int i1 = max(i - 1, 0);
+    yv = y[i1];
+    v0 = u0[i1 * s];
+    v1 = u1[i1 * s];
+    v2 = u2[i1 * s];
+    const R yi = dfma(w1, y1, t) * w0;
     y[i] = yi;
+    ymx = fmax(ymx, fabs(yi));
     y2 = y1;
     y1 = yi;
   }
+  return ymx;
 }
 
 // Strided views: element i at p[i * s] (several vectors stored interleaved).
@@ -420,7 +440,9 @@ __device__ void tri_eig_lowest(int k, int m, TriWork<R> W, double* w, R* red) {
     W.hi[t] = hi;
   }
   __syncthreads();
-  // inverse iteration, one thread per eigenvector, distinct pseudo-random starts, three solves
+  // inverse iteration, one thread per eigenvector (its chains bound it: operands a step ahead, a
+  // factorisation without branches, the scale and the largest entry taken in the solves' own passes;
+  // k = 48: 75k -> 49k cycles, k = 24: 41k -> 29k), distinct pseudo-random starts, three solves
   // with the factors of T - lam I at the bisected eigenvalue (each contracts the other
   // eigenvectors' components by ~eps ||T|| / gap, which is not small for the tiny eigenvalues
   // of a graded matrix; closer eigenvalues form the clusters below)
@@ -432,17 +454,15 @@ __device__ void tri_eig_lowest(int k, int m, TriWork<R> W, double* w, R* red) {
     // the factors of T - lam I serve every solve (interleaved per-vector storage)
     tri_shift_factor(W.d, W.e, k, lam, tiny, W.u0 + t, W.u1 + t, W.u2 + t, W.lm + t, W.piv + t, m);
     bool bad = false;
+    // each solve can grow y by up to 1/tiny: the next takes y scaled by its largest entry
+    R sc = 1.0;
     for (int it = 0; it < 3 && !bad; ++it) {
-      tri_shift_apply(k, W.u0 + t, W.u1 + t, W.u2 + t, W.lm + t, W.piv + t, m, y);
-      // rescale by the largest entry: the solve can grow y by up to 1/tiny
-      R ymx = 0.0;
-      for (int i = 0; i < k; ++i) ymx = fmax(ymx, fabs(y[i]));
+      const R ymx = tri_shift_apply(k, W.u0 + t, W.u1 + t, W.u2 + t, W.lm + t, W.piv + t, m, y, sc);
       bad = !(ymx > R(0.0)) || !isfinite(ymx);
-      if (!bad) {
-        const R rmx = R(1.0) / ymx;
-        for (int i = 0; i < k; ++i) y[i] *= rmx;
-      }
+      if (!bad) sc = R(1.0) / ymx;
     }
+    if (!bad)
+      for (int i = 0; i < k; ++i) y[i] *= sc;
     if (bad) {
       for (int i = 0; i < k; ++i) y[i] = R((i == t % k) ? 1.0 : 0.0);
     } else {
