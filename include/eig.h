@@ -60,9 +60,10 @@ typedef enum {
 } eig_method;
 
 /* Device layout of an SpMM plan's copy of H (all compute the same Y = H X).
- * MIRRORED: the plan expands the stored triangle into both triangles on the device (8-row
- *   groups of 64-column tiles, 1-byte column indices); the kernel only gathers.  About twice
- *   the matrix bytes of HALF, and the fastest on sm_103a.
+ * MIRRORED: the plan expands the stored triangle into both triangles on the device (row streams:
+ *   one lane per row, 2-byte column indices); the kernel only gathers.  About twice the matrix
+ *   bytes of HALF, and the fastest on sm_103a.  FP64 values with n < 65536 take streams without
+ *   row blocks and panels; the layout reported is the same.
  * HALF: the stored triangle only (tile chunks); each stored entry is applied as both H_ij and
  *   H_ji, the transposed half through per-tile scratch and a fixed-order reduction.
  * CSR: the CSR copy itself, read by a reference kernel (no tiled copy is built).
@@ -164,7 +165,8 @@ EIG_API eig_status eig_spmm_cheb(void* plan, const void* X, void* Y, int nb, eig
  * n x nb of vec_type (F32 or F64), nb <= 64; G: device FP64 nb x nb (row-major).  FP32 inputs:
  * products in FP32, 32-row partial sums accumulated in double-float (two FP32 words), CTA
  * partials in FP64, fixed-order reduction (bitwise reproducible).  Per-call scratch is taken
- * stream-ordered (cudaMallocAsync) and released on the same stream. */
+ * and released stream-ordered (cudaMallocFromPoolAsync, cudaFreeAsync) from a pool of the library's
+ * own, one per device, which keeps up to 32 MiB of freed scratch. */
 EIG_API eig_status eig_gram(const void* A, const void* B, int64_t n, int nb, eig_dtype vec_type, double* G,
                             void* stream);
 
