@@ -1398,7 +1398,7 @@ struct DirectArgs {
   int sms;
 };
 constexpr int kDirectWarps = 4;
-// Four doubles (32 bytes, one sector) in one load.
+// Four doubles (32 bytes, one sector) in one load; p 32-byte aligned.
 __device__ __forceinline__ Vec<double, 4> ld_sector(const double* p) {
   Vec<double, 4> r;
   asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
@@ -1406,7 +1406,9 @@ __device__ __forceinline__ Vec<double, 4> ld_sector(const double* p) {
   return r;
 }
 
-template <int NB, bool CHEB>
+// SECTOR (NB = 4): every gathered piece starts on a 32-byte boundary.  The products' inputs are only
+// aligned to 16 bytes, and a 32-byte load from such an address faults, so the host looks at X.
+template <int NB, bool CHEB, bool SECTOR>
 __global__ void __launch_bounds__(kDirectWarps * 32, 4)
 k_spmm_direct(const __grid_constant__ DirectArgs a, const double* __restrict__ X, double* __restrict__ Y, int ld,
               int col0, int slices, const __grid_constant__ MirrorEpi epi) {
@@ -1450,14 +1452,18 @@ k_spmm_direct(const __grid_constant__ DirectArgs a, const double* __restrict__ X
 #pragma unroll
     for (int k = 0; k < kBS; ++k) {
       const int64_t c = (k & 1) ? (c4[k >> 1] >> 16) : (c4[k >> 1] & 0xFFFFu);
-      if constexpr (NB == 4) {
+      if constexpr (SECTOR) {
+        static_assert(NB == 4, "a piece is one sector");
         Vec<double, 4> t;
         t.zero();
         if (b * kBS + k < len) t = ld_sector(Xc + c * ld);
         x[k][0].v[0] = t.v[0]; x[k][0].v[1] = t.v[1]; x[k][1].v[0] = t.v[2]; x[k][1].v[1] = t.v[3];
       } else {
-        x[k][0].zero();
-        if (b * kBS + k < len) x[k][0] = VecIO<double, VEC>::ld(Xc + c * ld);
+#pragma unroll
+        for (int j = 0; j < NCH; ++j) {
+          x[k][j].zero();
+          if (b * kBS + k < len) x[k][j] = VecIO<double, VEC>::ld(Xc + c * ld + j * VEC);
+        }
       }
     }
     if (b + 1 < nb) load(b + 1);
@@ -1615,11 +1621,14 @@ static eig_status rs_launch(SpmmPlan* P, const T* X, T* Y, int ld, int col0, con
   return EIG_OK;
 }
 
-// Columns [col0, col0 + nb) of a direct plan's product, in slices of at most four.
+// Columns [col0, col0 + nb) of a direct plan's product, in slices of at most four.  Slices of four
+// start on 32-byte boundaries when X does (ld and col0 are then multiples of four); an X that is only
+// 16-byte aligned is gathered in 16-byte pieces.
 template <int NB, bool CHEB>
 static eig_status direct_launch(SpmmPlan* P, const double* X, double* Y, int ld, int col0, const MirrorEpi& epi,
                                 cudaStream_t st) {
   constexpr int NS = NB < 4 ? NB : 4;
+  const bool sector = NS == 4 && (reinterpret_cast<uintptr_t>(X + col0) & 31u) == 0 && ld % 4 == 0;
   DirectArgs a;
   a.n = P->n;
   a.split = P->m_dsplit;
@@ -1631,8 +1640,9 @@ static eig_status direct_launch(SpmmPlan* P, const double* X, double* Y, int ld,
   a.bval = P->m_bval.as<double>();
   a.sms = num_sms();
   const int tasks = a.nw * (NB / NS);
-  k_spmm_direct<NS, CHEB><<<(unsigned)((tasks + kDirectWarps - 1) / kDirectWarps), kDirectWarps * 32, 0, st>>>(
-      a, X, Y, ld, col0, NB / NS, epi);
+  auto kern = sector ? k_spmm_direct<NS, CHEB, NS == 4> : k_spmm_direct<NS, CHEB, false>;
+  kern<<<(unsigned)((tasks + kDirectWarps - 1) / kDirectWarps), kDirectWarps * 32, 0, st>>>(a, X, Y, ld, col0, NB / NS,
+                                                                                           epi);
   EIG_LAUNCH_CHECK(CHEB ? "k_spmm_direct_cheb" : "k_spmm_direct");
   return EIG_OK;
 }

@@ -160,6 +160,40 @@ def test_spmm_direct_edges(n, nb):
     P.close()
 
 
+# FP64 blocks on 16-byte but not on 32-byte boundaries: legal (rows move in pieces of at most 16 bytes), and
+# the direct plans' gathers must then not take 32 bytes at once.  Each of X, Y and Qp is moved by itself
+# and all together; the sums are those of the aligned call.
+@pytest.mark.parametrize("n", [33, 2500])
+@pytest.mark.parametrize("nb", [2, 4, 8, 16, 32])
+def test_spmm_direct_16_byte_alignment(n, nb):
+    import oracle as O
+    from gen import ci_matrix, random_block
+    from gen.synth import CSRUpper
+    from paper_2305_15552_gb300 import binding as B
+
+    def moved(a, by):
+        v = torch.empty(a.size + by, dtype=torch.float64, device="cuda")[by:].view(a.shape)
+        v.copy_(torch.tensor(a))
+        assert v.data_ptr() % 32 == 8 * by
+        return v
+
+    H = ci_matrix(n, 30, 64, seed=5, storage="f64")
+    Xe, Qe = random_block(n, nb, seed=6), random_block(n, nb, seed=7)
+    Ha = CSRUpper(n=n, rowptr=H.rowptr, col=H.col, val=np.abs(H.val), storage="f64")
+    Yr, bound = O.sym_upper_matmul(H, Xe), O.sym_upper_matmul(Ha, np.abs(Xe))
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y0 = P.spmm(moved(Xe, 0))
+    # one rounding per multiply-add, rows of at most 300
+    assert np.all(np.abs(Y0.cpu().numpy() - Yr) <= 300 * 2.0 ** -53 * bound + 1e-300)
+    act = torch.tensor([j % 3 != 1 for j in range(nb)], dtype=torch.int32, device="cuda")
+    Z0 = P.spmm_cheb(moved(Xe, 0), 0.5, 2.0, moved(Qe, 0), act) if nb >= 8 else None
+    for bx, by, bq in [(2, 0, 0), (0, 2, 0), (0, 0, 2), (2, 2, 2)]:
+        assert torch.equal(P.spmm(moved(Xe, bx), moved(Xe, by)), Y0)
+        if nb >= 8:
+            assert torch.equal(P.spmm_cheb(moved(Xe, bx), 0.5, 2.0, moved(Qe, bq), act, Y=moved(Qe, by)), Z0)
+    P.close()
+
+
 # plan construction where it can go wrong: rows of more than 256 entries in a panel, row blocks of more
 # than 32 upper tiles (two counting groups), a tile with few rows of many entries, columns whose entries
 # all fall into one class mod 8, last row block and column block ragged
