@@ -58,7 +58,9 @@ __global__ void k_row_scan(int64_t n, int64_t nnz, int R, int C, int64_t words_p
       const bool in = q0 + 32 * u + lane < b;
       const int32_t up = __shfl_up_sync(0xffffffffu, c, 1);
       const int64_t prev = lane == 0 ? last : (int64_t)up;
-      const bool good = in && c > prev && c < n;
+      // its own range too, not only the order: prev may itself be invalid, and two negative columns in
+      // ascending order must not reach the bitmap
+      const bool good = in && c > prev && c >= i && c < n;
       ok = ok && (!in || good);
       if (good) {
         const unsigned cb = CC ? (unsigned)CC : (unsigned)C, J = (unsigned)c / cb;

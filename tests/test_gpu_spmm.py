@@ -187,6 +187,25 @@ def test_invalid_csr_rejected():
     assert e.value.status == binding.EIG_EINVAL
 
 
+# two columns out of range in ascending order (the second one follows a smaller one): at a row's start, in
+# its middle, across the 32 and 128 entries that the check reads at a time, at its end
+@pytest.mark.parametrize("layout,C", [("auto", 0), ("mirrored", 64), ("half", 64), ("csr", 32)])
+@pytest.mark.parametrize("at", [0, 1, 31, 127, 148])
+@pytest.mark.parametrize("pair", [(-5, -3), (-2 ** 31, -2 ** 31 + 64), (-1, 3), (500, 501), (2 ** 31 - 2, 2 ** 31 - 1)])
+def test_invalid_csr_consecutive_columns(layout, C, at, pair):
+    from paper_2305_15552_gb300 import binding
+    n, r, m = 500, 10, 150
+    rowptr = np.concatenate([np.arange(r + 1), np.arange(r, n) + m])
+    col = np.concatenate([np.arange(r), np.arange(r, r + m), np.arange(r + 1, n)]).astype(np.int32)
+    assert rowptr.size == n + 1 and col.size == rowptr[-1]
+    val = np.ones(col.size, np.float32)
+    _plan(CSRUpper(n, rowptr, col.copy(), val, "f32"), col_block=C, layout=layout).close()
+    col[r + at:r + at + 2] = pair
+    with pytest.raises(binding.EigError) as e:
+        _plan(CSRUpper(n, rowptr, col, val, "f32"), col_block=C, layout=layout)
+    assert e.value.status == binding.EIG_EINVAL
+
+
 @pytest.fixture(scope="module")
 def bench_matrix():
     return ci_matrix(2_000_000, 400, 256, seed=1, storage="f32")
