@@ -36,9 +36,14 @@ struct ScratchPools {
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
       uint64_t keep = 32u << 20;
+      // the first call may come while this or another thread captures a stream, which creating a pool in
+      // the thread's own capture mode would invalidate; nothing here enters the capture
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
       if (cudaMemPoolCreate(&pool[dev], &props) != cudaSuccess) pool[dev] = nullptr;
       else cudaMemPoolSetAttribute(pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
       cudaGetLastError();
+      cudaThreadExchangeStreamCaptureMode(&mode);
     }
     return pool[dev];
   }

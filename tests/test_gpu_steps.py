@@ -168,3 +168,35 @@ def test_rmm_diis_matches_oracle(s):
         ref = O.diis_coefficients(rs[j])
         np.testing.assert_allclose(al[j, :s], ref, rtol=1e-8, atol=1e-10)
         assert abs(al[j, :s].sum() - 1) < 1e-12
+
+
+FIRST_CALL_UNDER_CAPTURE = """
+import torch
+from paper_2305_15552_gb300 import binding as B
+lib = B.load()
+A = torch.randn(5000, 8, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+G = torch.zeros(8, 8, device="cuda", dtype=torch.float64)
+s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+torch.cuda.synchronize()
+with torch.cuda.graph(graph, stream=s, capture_error_mode="{mode}"):
+    rc = lib.eig_gram(A.data_ptr(), A.data_ptr(), 5000, 8, B.EIG_F32, G.data_ptr(), s.cuda_stream)
+assert rc == B.EIG_OK, (rc, lib.eig_last_cuda_error())
+for _ in range(2):
+    G.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(G, B.gram(A, A))
+"""
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+def test_first_step_call_of_a_process_under_capture(mode):
+    """The first step call of a process creates the library's scratch pool; made while the stream is
+    captured, in any capture mode, it must be recorded like any other (a process of its own each)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", FIRST_CALL_UNDER_CAPTURE.replace("{mode}", mode)], cwd=root,
+                       capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0, p.stderr[-2000:]
