@@ -1136,11 +1136,11 @@ __device__ __forceinline__ void stage_df_rows(unsigned char* xs, const double* _
                                               int npt, int64_t n) {
   constexpr int PPR = NB / 2, U = 8;   // pieces per row, loads in flight
   const int total = npt * kMC * PPR;
-  for (int i0 = threadIdx.x; i0 < total; i0 += U * blockDim.x) {
+  for (int i0 = threadIdx.x; i0 < total; i0 += U * kW * 32) {
     double2 x[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * blockDim.x;
+      const int i = i0 + u * kW * 32;
       x[u] = make_double2(0.0, 0.0);
       if (i < total) {
         const int64_t row = (int64_t)tcol[i / (kMC * PPR)] * kMC + i / PPR % kMC;
@@ -1149,7 +1149,7 @@ __device__ __forceinline__ void stage_df_rows(unsigned char* xs, const double* _
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * blockDim.x;
+      const int i = i0 + u * kW * 32;
       if (i >= total) break;
       const float h0 = __double2float_rn(x[u].x), h1 = __double2float_rn(x[u].y);
       reinterpret_cast<float4*>(xs)[i] = make_float4(h0, h1, __double2float_rn(x[u].x - (double)h0),
@@ -1219,7 +1219,8 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
     } else if (DF && NB >= 2 && ld == NB) {
       if constexpr (DF && NB >= 2) stage_df_rows<NB>(xs, X, a.tcol + t0, npt, a.n);
     } else {
-      for (int64_t i = tid; i < (int64_t)npt * kMC * NB; i += blockDim.x) {
+      // a whole CTA (the host does not split row blocks here): a constant stride
+      for (int64_t i = tid; i < (int64_t)npt * kMC * NB; i += kW * 32) {
         const int t = (int)(i / (kMC * NB));
         const int rr = (int)((i / NB) % kMC), e = (int)(i % NB);
         const int64_t row = (int64_t)a.tcol[t0 + t] * kMC + rr;
