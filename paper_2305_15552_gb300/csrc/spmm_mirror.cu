@@ -81,7 +81,8 @@ __device__ __forceinline__ int tile_index(const uint32_t* slot, const int32_t* t
 // in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper entries of each
 // column (integer atomics in shared memory: order independent); the largest total of a tile; and, in the
 // bitmap of the full matrix, the transposed tiles (64 rows of this row block as a column block of the
-// row block that holds the tile's columns).
+// row block that holds the tile's columns).  A group takes up each row where the group before it left
+// it, so that a row is read once however many groups there are.
 constexpr int kCountTiles = 32;
 __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ col,
@@ -93,8 +94,10 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
   __shared__ int32_t s_tc[kCountTiles];
   __shared__ uint32_t s_slot[256];          // tile column and index, at the column mod 256 (one of them)
   __shared__ unsigned s_sub[kCountTiles];   // bit q: the 64 rows q have strictly-upper entries in the tile
+  __shared__ int32_t s_next[kMR];           // per row: offset of the first chunk that the groups so far left
   const int64_t I = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  s_next[tid] = 0;
   const int64_t t0 = tile_ptr[I], t1 = tile_ptr[I + 1];
   for (int64_t g0 = t0; g0 < t1; g0 += kCountTiles) {
     const int nt = (int)min64(kCountTiles, t1 - g0);
@@ -113,10 +116,12 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
       const int64_t r = I * kMR + lr;
       if (r >= n) break;
       const int64_t e0 = rowptr[r], e1 = rowptr[r + 1];
-      int32_t before = -1;   // tile column of the entry before the chunk
-      bool past = false;
-      for (int64_t q0 = e0; q0 < e1 && !past; q0 += 128) {
-        int32_t cs[4];
+      // tile column of the entry before the chunk, where it matters: an entry before the first chunk
+      // belongs to an earlier group
+      int32_t before = -1;
+      int64_t q0 = e0 + s_next[lr];
+      for (; q0 < e1; q0 += 128) {
+        int32_t cs[4], top = -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u) cs[u] = q0 + 32 * u + lane < e1 ? col[q0 + 32 * u + lane] : INT32_MAX;
 #pragma unroll
@@ -134,9 +139,11 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
             if ((int64_t)c != r) atomicAdd(&s_cnt[lo][c - J * kMC], 1);
           }
           before = __shfl_sync(0xffffffffu, J, 31);
+          if (c != INT32_MAX) top = J;
         }
-        past = before > last;   // also after the row's end (INT32_MAX)
+        if (__any_sync(0xffffffffu, top > last)) break;   // the next group starts with this chunk
       }
+      if (lane == 0) s_next[lr] = (int32_t)(min64(q0, e1) - e0);
     }
     __syncthreads();
     for (int t = w; t < nt; t += kW) {

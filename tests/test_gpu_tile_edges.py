@@ -232,3 +232,85 @@ def test_plan_streams_edges(kind, val, dt):
     # rows of at most n terms: one rounding of the running sum per term in FP32, 2^-44 in double-float
     eps = 2.0 ** -24 if dt == torch.float32 else 2.0 ** -44
     assert np.all(np.abs(Y - O.sym_upper_matmul(H, Xe)) <= n * eps * bound + 1e-300)
+
+
+def _many_tiles(kind, n, rng):
+    """Upper triangles whose row blocks have up to n / 64 tiles: row, column lists."""
+    i = np.arange(n)
+    r, c = [i], [i]
+    if kind == "scattered":                 # a handful of entries per tile
+        a, b = rng.integers(0, n, 30 * n), rng.integers(0, n, 30 * n)
+        r += [np.minimum(a, b)]
+        c += [np.maximum(a, b)]
+    elif kind == "one_per_tile":            # the last column of every tile, the same for all rows
+        for j in range(63, n, 64):
+            k = i[i < j]
+            r += [k]
+            c += [np.full(k.size, j)]
+    elif kind == "dense_rows":              # lengths around multiples of the 128 entries read at a time
+        for x, m in [(3, n), (4, n), (300, 128), (301, 129), (302, 127), (303, 4096), (n - 400, 400)]:
+            m = min(m, n - x)
+            r += [np.full(m, x)]
+            c += [np.arange(x, x + m)]
+    else:                                   # "gaps": runs of 200 entries, 40 tiles without any between them
+        for x in range(0, n, 37):
+            k = np.concatenate([np.arange(q, min(q + 200, n)) for q in range(x, n, 64 * 40)])
+            r += [np.full(k.size, x)]
+            c += [k]
+    key = np.unique(np.concatenate(r) * n + np.concatenate(c))
+    return key // n, key % n
+
+
+# row blocks of many tiles: several groups of 32 tiles in the column counts, rows left in the middle of a
+# chunk of 128 entries and taken up again, panels by the dozen; small integers, so that every product is
+# exact in any order
+@pytest.mark.parametrize("kind", ["scattered", "one_per_tile", "dense_rows", "gaps"])
+@pytest.mark.parametrize("val,dt", [("f32", torch.float32), ("bf16", torch.float32), ("f32", torch.float64),
+                                    ("f64", torch.float64)])
+@pytest.mark.parametrize("n", [9 * 256 + 37, 70000])
+def test_plan_many_tiles_exact(kind, val, dt, n):
+    import oracle as O
+    from gen.synth import CSRUpper, round_to_storage
+    from paper_2305_15552_gb300 import binding as B
+    if kind == "one_per_tile" and n > 10000:
+        n = 20480
+    rng = np.random.default_rng(n)
+    r, c = _many_tiles(kind, n, rng)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(r, minlength=n), out=rowptr[1:])
+    H = CSRUpper(n=n, rowptr=rowptr, col=c.astype(np.int32), val=round_to_storage(
+        rng.integers(1, 4, r.size).astype(np.float64), val), storage=val)
+    X = torch.tensor(rng.integers(-3, 4, (n, 8)), dtype=dt, device="cuda")
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y = P.spmm(X).double().cpu().numpy()
+    P.close()
+    # sums of at most n products of magnitude 9: integers below 2^24
+    assert 9 * n < 2 ** 24
+    assert np.array_equal(Y, O.sym_upper_matmul(H, X.double().cpu().numpy()))
+
+
+def test_plan_time_of_a_dense_row():
+    """One dense row among 2M (31,250 tiles in one row block, 977 groups): the row is read once, not
+    once per group.  Read once, the plan takes some tens of ms; once per group, 2 s and more."""
+    import time
+    from gen.synth import CSRUpper
+    from paper_2305_15552_gb300 import binding as B
+    n = 2_000_000
+    rowptr = np.concatenate([[0], np.arange(n) + n]).astype(np.int64)
+    col = np.concatenate([np.arange(n), np.arange(1, n)]).astype(np.int32)
+    H = CSRUpper(n=n, rowptr=rowptr, col=col, val=np.ones(col.size, np.float32), storage="f32")
+    dev = tuple(torch.tensor(a, device="cuda") for a in (H.rowptr, H.col, H.val))
+    best = np.inf
+    for _ in range(2):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        P = B.SpmmPlan(H, device_arrays=dev, layout="mirrored", copy=False)
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t)
+        x = torch.ones(n, 1, device="cuda")
+        y = P.spmm(x).cpu().numpy()[:, 0]
+        P.close()
+    want = np.full(n, 2.0)
+    want[0] = n
+    assert np.array_equal(y, want)
+    assert best < 1.0, best
