@@ -268,7 +268,7 @@ eig_status spmm_plan_build(SpmmPlan* P, const eig_csr_upper* H, int R, int C, in
   if (want_mirror && layout == EIG_LAYOUT_AUTO) {
     size_t fr = 0, tot = 0;
     EIG_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
-    want_mirror = mirror_bytes_estimate(P) < fr / 10 * 8;
+    want_mirror = mirror_bytes_estimate(P) < fr / 10 * 8 && mirror_tiles_bytes(P) < fr;
   }
   if (want_mirror) {   // gathers only: no transpose schedule
     EIG_TRY(spmm_plan_build_mirror(P, h_ptr, h_col, tmp, st));

@@ -101,6 +101,9 @@ eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tpt
                                   const std::vector<int32_t>& h_tcol, PlanTemps& tmp, cudaStream_t st);
 // Device bytes the mirrored layout needs while it is built (estimate).
 size_t mirror_bytes_estimate(const SpmmPlan* P);
+// Those of the arrays over its tiles and the lower CSR, which are there together before the streams are
+// (more than the estimate only where tiles hold a handful of entries).
+size_t mirror_tiles_bytes(const SpmmPlan* P);
 // Builds the tile-contiguous copy (called by spmm_plan_build).
 eig_status spmm_plan_build_tiled(SpmmPlan* P, int cap, cudaStream_t st);
 eig_status spmm_run(SpmmPlan* P, const void* X, void* Y, int nb, eig_dtype vt, cudaStream_t st);

@@ -57,11 +57,21 @@ constexpr int kBE = 32 * kBS;            // entries per block (32 lanes)
 constexpr int kPT = 24;                  // tiles per panel at most (<= 32: one lane stages one tile)
 constexpr int kPR = kPT * kMC;           // staged X rows per panel at most; 8 zero rows follow
 constexpr int kL2 = 6;                   // streamed blocks prefetched into L2 ahead of use
+constexpr int kDenseTile = 3000;         // mean stored entries of a tile (see dense_tiles)
 
 // ---------------------------------------------------------------------------------------
 // Plan: the strictly lower triangle as a CSR beside the upper one, built from U without sorting and
 // without atomics on values.  A row of H is its row of the lower CSR, then its row of U.
 // ---------------------------------------------------------------------------------------
+
+// First of the ascending c[a, b) that is at least lim.
+__device__ __forceinline__ int64_t first_from(const int32_t* __restrict__ c, int64_t a, int64_t b, int64_t lim) {
+  while (a < b) {
+    const int64_t m = (a + b) >> 1;
+    if ((int64_t)c[m] < lim) a = m + 1; else b = m;
+  }
+  return a;
+}
 
 // Index of tile column J among the nt <= 32 ascending columns tc, which hold it: slot[J mod 256] names
 // one tile (J < 2^25 in the upper bits, its index in the lower five); where it names another, by search.
@@ -77,8 +87,8 @@ __device__ __forceinline__ int tile_index(const uint32_t* slot, const int32_t* t
 }
 
 // CTA per row block, warp per row (32 rows each), the row block's upper tiles (256 rows x 64 columns) in
-// groups of kCountTiles.  Per tile: seg[t * 256 + row], the offset in its row of the row's first entry
-// in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper entries of each
+// groups of kCountTiles.  Per tile: seg[t * 256 + row] (unless seg is null), the offset in its row of the
+// row's first entry in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper entries of each
 // column (integer atomics in shared memory: order independent); the largest total of a tile; and, in the
 // bitmap of the full matrix, the transposed tiles (64 rows of this row block as a column block of the
 // row block that holds the tile's columns).  A group takes up each row where the group before it left
@@ -131,7 +141,7 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
           if (c != INT32_MAX && J >= first && J <= last) {
             const int lo = tile_index(s_slot, s_tc, nt, J);
             if ((lane == 0 ? before : up) != J) {
-              seg[(g0 + lo) * kMR + lr] = (int32_t)(q0 + 32 * u + lane - e0);
+              if (seg) seg[(g0 + lo) * kMR + lr] = (int32_t)(q0 + 32 * u + lane - e0);
               // a row whose only entry here is its diagonal has nothing strictly upper, but the tile
               // then belongs to this row block already
               if ((s_sub[lo] >> (lr / kMC) & 1u) == 0u) atomicOr(&s_sub[lo], 1u << (lr / kMC));
@@ -372,6 +382,47 @@ __global__ void __launch_bounds__(kMR, 6) k_mir_lower(int64_t n, const int64_t* 
   }
 }
 
+// The same for tiles of fewer entries (see dense_tiles): thread per row, which searches its row for the tile's
+// first column instead of reading an offset kept per (tile, row), and writes each entry to its place.
+template <typename V>
+__global__ void __launch_bounds__(kMR) k_mir_lower_few(int64_t n, const int64_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ col, const V* __restrict__ val,
+                                                       const int32_t* __restrict__ tile_rb,
+                                                       const int32_t* __restrict__ tile_cb,
+                                                       const int32_t* __restrict__ off,
+                                                       const int64_t* __restrict__ lptr, int32_t* __restrict__ lcol,
+                                                       V* __restrict__ lval) {
+  constexpr int NW = kMR / 32;
+  __shared__ unsigned bits[NW][kMC];   // bit b of word [w][j]: entry (row 32 w + b, column j)
+  const int64_t t = blockIdx.x;
+  const int tid = threadIdx.x, w = tid >> 5;
+  for (int i = tid; i < NW * kMC; i += kMR) (&bits[0][0])[i] = 0u;
+  const int64_t r = (int64_t)tile_rb[t] * kMR + tid, cb0 = (int64_t)tile_cb[t] * kMC;
+  int64_t a = 0, b = 0;
+  if (r < n) {
+    b = rowptr[r + 1];
+    a = first_from(col, rowptr[r], b, cb0);
+  }
+  __syncthreads();
+  int64_t e = a;   // past the row's last entry in the tile
+  for (; e < b; ++e) {
+    const int64_t c = col[e];
+    if (c >= cb0 + kMC) break;
+    if (c != r) atomicOr(&bits[w][c - cb0], 1u << (tid & 31));
+  }
+  __syncthreads();
+  for (int64_t k = a; k < e; ++k) {
+    const int64_t c = col[k];
+    if (c == r) continue;
+    const int j = (int)(c - cb0);
+    int rank = __popc(bits[w][j] & ((1u << (tid & 31)) - 1u));
+    for (int q = 0; q < w; ++q) rank += __popc(bits[q][j]);
+    const int64_t pos = lptr[c] + off[t * kMC + j] + rank;
+    lcol[pos] = (int32_t)r;
+    lval[pos] = val[k];
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Plan: the row streams
 // ---------------------------------------------------------------------------------------
@@ -380,15 +431,6 @@ __global__ void __launch_bounds__(kMR, 6) k_mir_lower(int64_t n, const int64_t* 
 __device__ __forceinline__ int64_t panel_last_cb(const int32_t* __restrict__ pt0, const int32_t* __restrict__ pnt,
                                                  const int32_t* __restrict__ tcol, int64_t p) {
   return pnt[p] > 0 ? (int64_t)tcol[pt0[p] + pnt[p] - 1] : -1;
-}
-
-// First of the ascending c[a, b) that is at least lim.
-__device__ __forceinline__ int64_t first_from(const int32_t* __restrict__ c, int64_t a, int64_t b, int64_t lim) {
-  while (a < b) {
-    const int64_t m = (a + b) >> 1;
-    if ((int64_t)c[m] < lim) a = m + 1; else b = m;
-  }
-  return a;
 }
 
 // Thread per row: entries the row has in each panel of its row block, and those of them left of the
@@ -735,10 +777,24 @@ eig_status direct_fill(SpmmPlan* P, const int64_t* lptr, const int32_t* lcol, co
   return EIG_OK;
 }
 
+// Arrays over the upper tiles, which a plan needs until its lower CSR is built: tile row and column blocks,
+// tiles by column block; entries per (tile, column) and their offsets; offsets per (tile, row), or null.
+struct TileTemps {
+  DevBuf mem, rb, cb, jptr, jt, cnt, off, seg, most;
+};
+
+// Tiles that hold many entries on average (of 16,384): their lower part is built by k_mir_lower, with an
+// offset kept per (tile, row).  Else k_mir_lower_few searches the rows and no offsets are kept: 1 KB a tile
+// would be several times the matrix where tiles hold a handful of entries, and the CTAs of nearly empty tiles
+// would mostly set themselves up.  A whole plan with k_mir_lower / with k_mir_lower_few, FP32, ms, by mean
+// entries of a tile: 8: 32.7 / 20.4, 156: 18.8 / 12.8, 1009: 5.26 / 4.74, 2446: 3.94 / 3.93, 3393 (n = 1M, 300
+// a row): 8.56 / 9.05.
+bool dense_tiles(const SpmmPlan* P) { return P->nnz >= kDenseTile * P->n_tiles; }
+
 template <typename V>
-eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* tile_cb, int64_t n_up_tiles,
-                          const int64_t* jt_ptr, const int32_t* jt_tile, int32_t* cnt, int32_t* off, int32_t* seg, PlanTemps& tmp,
-                          cudaStream_t st) {
+eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStream_t st) {
+  const int32_t *tile_rb = tiles.rb.as<int32_t>(), *tile_cb = tiles.cb.as<int32_t>();
+  const int64_t n_up_tiles = P->n_tiles;
   const int64_t n = P->n;
   const int tb = 256;
   const int64_t gb = (n + tb - 1) / tb;
@@ -747,13 +803,15 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   const DevBuf &lower = tmp.lower, &lptr = tmp.lptr;
   unsigned* bitmap = tmp.bitmap.as<unsigned>();
   const int64_t nRB = P->nRB, wpr = (P->nCB + 31) / 32;
-  int* most_d = seg + std::max<int64_t>(n_up_tiles, 1) * kMR;
+  int32_t *cnt = tiles.cnt.as<int32_t>(), *off = tiles.off.as<int32_t>(), *seg = tiles.seg.as<int32_t>();
+  int* most_d = tiles.most.as<int>();
   EIG_CUDA_TRY(cudaMemsetAsync(most_d, 0, 4, st));
-  EIG_CUDA_TRY(cudaMemsetAsync(seg, 0x7F, std::max<int64_t>(n_up_tiles, 1) * kMR * 4, st));   // "none"
+  if (seg) EIG_CUDA_TRY(cudaMemsetAsync(seg, 0x7F, tiles.seg.bytes, st));   // "none"
   k_mir_colcounts<<<(unsigned)nRB, kMR, 0, st>>>(n, P->rowptr, P->col, P->tile_ptr.as<int64_t>(),
                                                  P->tile_col.as<int32_t>(), wpr, seg, cnt, bitmap, most_d);
   EIG_LAUNCH_CHECK("k_mir_colcounts");
-  k_mir_coloffsets<<<(unsigned)gb, tb, 0, st>>>(n, jt_ptr, jt_tile, cnt, off, lower.as<int64_t>());
+  k_mir_coloffsets<<<(unsigned)gb, tb, 0, st>>>(n, tiles.jptr.as<int64_t>(), tiles.jt.as<int32_t>(), cnt, off,
+                                                lower.as<int64_t>());
   EIG_LAUNCH_CHECK("k_mir_coloffsets");
   EIG_TRY(exclusive_scan(lower.as<int64_t>(), n, lptr.as<int64_t>(), tmp.sums.as<int64_t>(), st));
   int64_t lnnz = 0;
@@ -768,7 +826,11 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   EIG_TRY(full.reserve(DevBuf::part(b_lcol) + DevBuf::part(b_lval)));
   lcol.borrow(full, b_lcol, &at);
   lval.borrow(full, b_lval, &at);
-  if (most > 0) {
+  if (most > 0 && !seg) {
+    k_mir_lower_few<V><<<(unsigned)n_up_tiles, kMR, 0, st>>>(n, P->rowptr, P->col, val, tile_rb, tile_cb, off,
+                                                             lptr.as<int64_t>(), lcol.as<int32_t>(), lval.as<V>());
+    EIG_LAUNCH_CHECK("k_mir_lower_few");
+  } else if (most > 0) {
     const int cap = (most + 15) / 16 * 16;
     const size_t sm = (size_t)cap * (sizeof(V) + 1);
     if (sm > 40 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_mir_lower<V>, sm));
@@ -785,6 +847,7 @@ eig_status rowstream_fill(SpmmPlan* P, const int32_t* tile_rb, const int32_t* ti
   std::vector<int64_t> h_tptr;
   std::vector<int32_t> h_tcol;
   EIG_TRY(tile_lists_from_bitmap(nRB, wpr, bitmap, tmp.rb_cnt.as<int64_t>(), st, tmp.rb_ptr, P->m_tcol, h_tptr, h_tcol));
+  tiles.mem.release();   // the lists' copies waited for the kernels above; the streams may need the room
   std::vector<int32_t> rbp(nRB + 1, 0), pt0, pnt;
   for (int64_t I = 0; I < nRB; ++I) {
     const int64_t t0 = h_tptr[I], nt = h_tptr[I + 1] - t0;
@@ -1520,8 +1583,12 @@ size_t mirror_bytes_estimate(const SpmmPlan* P) {
   // lower CSR (temporary) + streams of 2-byte columns and values with ~5% padding
   const double fnnz = 2.0 * double(P->nnz);
   const double vb = double(dtype_size(P->val_type));
-  // and, while it is built, the rows' offsets in every upper tile
-  return (size_t)(0.5 * fnnz * (4.0 + vb) + 1.1 * fnnz * (2.0 + vb) + 64.0 * double(P->n) + 1536.0 * double(P->n_tiles));
+  return (size_t)(0.5 * fnnz * (4.0 + vb) + 1.1 * fnnz * (2.0 + vb) + 64.0 * double(P->n));
+}
+
+size_t mirror_tiles_bytes(const SpmmPlan* P) {
+  const size_t per_tile = 3 * 4 + 2 * kMC * 4 + (dense_tiles(P) ? kMR * 4 : 0);
+  return (size_t)P->n_tiles * per_tile + (size_t)P->nnz * (4 + dtype_size(P->val_type));
 }
 
 eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tptr,
@@ -1544,31 +1611,27 @@ eig_status spmm_plan_build_mirror(SpmmPlan* P, const std::vector<int64_t>& h_tpt
     for (int64_t t = 0; t < nt; ++t) jt[fill[tcb[t]]++] = (int32_t)t;
   }
   const size_t t4 = std::max<int64_t>(nt, 1) * 4;
-  DevBuf mem, d_trb, d_tcb, d_jptr, d_jt, cnt, off, seg;
+  const size_t b_seg = dense_tiles(P) ? t4 * kMR : 0;
+  TileTemps T;
   size_t at = 0;
-  EIG_TRY(mem.reserve(3 * DevBuf::part(t4) + DevBuf::part(jptr.size() * 8) + 2 * DevBuf::part(t4 * kMC) +
-                      DevBuf::part(t4 * kMR + 4)));
-  d_trb.borrow(mem, t4, &at);
-  d_tcb.borrow(mem, t4, &at);
-  d_jt.borrow(mem, t4, &at);
-  d_jptr.borrow(mem, jptr.size() * 8, &at);
-  cnt.borrow(mem, t4 * kMC, &at);
-  off.borrow(mem, t4 * kMC, &at);
-  seg.borrow(mem, t4 * kMR + 4, &at);
-  EIG_CUDA_TRY(cudaMemcpyAsync(d_trb.p, trb.data(), trb.size() * 4, cudaMemcpyHostToDevice, st));
-  EIG_CUDA_TRY(cudaMemcpyAsync(d_tcb.p, tcb.data(), tcb.size() * 4, cudaMemcpyHostToDevice, st));
-  EIG_CUDA_TRY(cudaMemcpyAsync(d_jptr.p, jptr.data(), jptr.size() * 8, cudaMemcpyHostToDevice, st));
-  EIG_CUDA_TRY(cudaMemcpyAsync(d_jt.p, jt.data(), jt.size() * 4, cudaMemcpyHostToDevice, st));
+  EIG_TRY(T.mem.reserve(3 * DevBuf::part(t4) + DevBuf::part(jptr.size() * 8) + 2 * DevBuf::part(t4 * kMC) +
+                        DevBuf::part(4) + DevBuf::part(b_seg)));
+  T.rb.borrow(T.mem, t4, &at);
+  T.cb.borrow(T.mem, t4, &at);
+  T.jt.borrow(T.mem, t4, &at);
+  T.jptr.borrow(T.mem, jptr.size() * 8, &at);
+  T.cnt.borrow(T.mem, t4 * kMC, &at);
+  T.off.borrow(T.mem, t4 * kMC, &at);
+  T.most.borrow(T.mem, 4, &at);
+  if (b_seg) T.seg.borrow(T.mem, b_seg, &at);
+  EIG_CUDA_TRY(cudaMemcpyAsync(T.rb.p, trb.data(), trb.size() * 4, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(T.cb.p, tcb.data(), tcb.size() * 4, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(T.jptr.p, jptr.data(), jptr.size() * 8, cudaMemcpyHostToDevice, st));
+  EIG_CUDA_TRY(cudaMemcpyAsync(T.jt.p, jt.data(), jt.size() * 4, cudaMemcpyHostToDevice, st));
   eig_status s;
-  if (P->val_type == EIG_F32)
-    s = rowstream_fill<float>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                              d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
-  else if (P->val_type == EIG_F64)
-    s = rowstream_fill<double>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                               d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
-  else
-    s = rowstream_fill<uint16_t>(P, d_trb.as<int32_t>(), d_tcb.as<int32_t>(), nt, d_jptr.as<int64_t>(),
-                                 d_jt.as<int32_t>(), cnt.as<int32_t>(), off.as<int32_t>(), seg.as<int32_t>(), tmp, st);
+  if (P->val_type == EIG_F32) s = rowstream_fill<float>(P, T, tmp, st);
+  else if (P->val_type == EIG_F64) s = rowstream_fill<double>(P, T, tmp, st);
+  else s = rowstream_fill<uint16_t>(P, T, tmp, st);
   EIG_TRY(s);
   P->mirrored = true;
   return EIG_OK;

@@ -314,3 +314,38 @@ def test_plan_time_of_a_dense_row():
     want[0] = n
     assert np.array_equal(y, want)
     assert best < 1.0, best
+
+
+def test_plan_memory_of_scattered_entries():
+    """1.2M tiles of 8 entries: the arrays over the tiles (0.6 GB) are gone before the streams (0.8 GB)
+    are built, and no offset is kept per (tile, row) (1.3 GB).  With 1.9 GB left on the device the mirrored
+    layout is built, and AUTO takes it."""
+    import oracle as O
+    from gen.synth import CSRUpper
+    from paper_2305_15552_gb300 import binding as B
+    n = 200_000
+    rng = np.random.default_rng(2)
+    a, b = rng.integers(0, n, 50 * n), rng.integers(0, n, 50 * n)
+    key = np.unique(np.concatenate([np.minimum(a, b) * n + np.maximum(a, b), np.arange(n) * n + np.arange(n)]))
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(key // n, minlength=n), out=rowptr[1:])
+    H = CSRUpper(n=n, rowptr=rowptr, col=(key % n).astype(np.int32), storage="f32",
+                 val=rng.integers(1, 4, key.size).astype(np.float32))
+    dev = tuple(torch.tensor(x, device="cuda") for x in (H.rowptr, H.col, H.val))
+    X = torch.tensor(rng.integers(-3, 4, (n, 8)), dtype=torch.float32, device="cuda")
+    Y = torch.empty_like(X)
+    B.SpmmPlan(H, device_arrays=dev, layout="mirrored", copy=False).close()      # code loaded
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - 1_900_000_000, dtype=torch.uint8, device="cuda")
+    try:
+        for layout in ("mirrored", "auto"):
+            P = B.SpmmPlan(H, device_arrays=dev, layout=layout, copy=False)
+            assert P.info()["layout"] == B.LAYOUTS["mirrored"]
+            assert P.info()["n_tiles"] > 1_100_000
+            P.spmm(X, Y)
+            P.close()
+            assert np.array_equal(Y.double().cpu().numpy(), O.sym_upper_matmul(H, X.double().cpu().numpy()))
+    finally:
+        del rest
+        torch.cuda.empty_cache()
