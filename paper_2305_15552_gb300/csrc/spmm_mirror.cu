@@ -64,6 +64,20 @@ constexpr int kDenseTile = 3000;         // mean stored entries of a tile (see d
 // without atomics on values.  A row of H is its row of the lower CSR, then its row of U.
 // ---------------------------------------------------------------------------------------
 
+// First of the ascending c[a, b) that is at least lim, expected near a.
+__device__ __forceinline__ int64_t first_near(const int32_t* __restrict__ c, int64_t a, int64_t b, int64_t lim) {
+  int64_t step = 1;
+  while (a < b && (int64_t)c[min64(a + step, b) - 1] < lim) {
+    a = min64(a + step, b);
+    step *= 2;
+  }
+  for (int64_t e = min64(a + step, b); a < e;) {
+    const int64_t m = (a + e) >> 1;
+    if ((int64_t)c[m] < lim) a = m + 1; else e = m;
+  }
+  return a;
+}
+
 // First of the ascending c[a, b) that is at least lim.
 __device__ __forceinline__ int64_t first_from(const int32_t* __restrict__ c, int64_t a, int64_t b, int64_t lim) {
   while (a < b) {
@@ -122,6 +136,7 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
     if (tid < nt) s_slot[s_tc[tid] & 255] = ((uint32_t)s_tc[tid] << 5) | tid;
     __syncthreads();
     const int32_t first = s_tc[0], last = s_tc[nt - 1];
+    const bool again = g0 + nt < t1;   // another group follows
     for (int lr = w; lr < kMR; lr += kW) {
       const int64_t r = I * kMR + lr;
       if (r >= n) break;
@@ -131,7 +146,7 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
       int32_t before = -1;
       int64_t q0 = e0 + s_next[lr];
       for (; q0 < e1; q0 += 128) {
-        int32_t cs[4], top = -1;
+        int32_t cs[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) cs[u] = q0 + 32 * u + lane < e1 ? col[q0 + 32 * u + lane] : INT32_MAX;
 #pragma unroll
@@ -149,11 +164,16 @@ __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t*
             if ((int64_t)c != r) atomicAdd(&s_cnt[lo][c - J * kMC], 1);
           }
           before = __shfl_sync(0xffffffffu, J, 31);
-          if (c != INT32_MAX) top = J;
         }
-        if (__any_sync(0xffffffffu, top > last)) break;   // the next group starts with this chunk
+        if (before > last) {   // also after the row's end (INT32_MAX)
+          bool more = false;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) more = more || (cs[u] != INT32_MAX && cs[u] / kMC > last);
+          if (again && !__any_sync(0xffffffffu, more)) q0 = e1;   // else the next group starts with this chunk
+          break;
+        }
       }
-      if (lane == 0) s_next[lr] = (int32_t)(min64(q0, e1) - e0);
+      if (again && lane == 0) s_next[lr] = (int32_t)(min64(q0, e1) - e0);
     }
     __syncthreads();
     for (int t = w; t < nt; t += kW) {
@@ -446,10 +466,12 @@ __global__ void k_rs_counts(int64_t n, const int64_t* __restrict__ lptr, const i
   const int lr = (int)(r - I * kMR);
   int64_t kl = lptr[r], ku = rowptr[r];
   const int64_t el = lptr[r + 1], eu = rowptr[r + 1];
+  const bool many = rbp[I + 1] - rbp[I] > 8;   // panels, with few entries of the row each
   for (int64_t p = rbp[I]; p < rbp[I + 1]; ++p) {
     const bool last = p + 1 == rbp[I + 1];
     const int64_t lim = (panel_last_cb(pt0, pnt, tcol, p) + 1) * kMC;   // first column past the panel
-    const int64_t nl = last ? el : first_from(lcol, kl, el, lim), nu = last ? eu : first_from(col, ku, eu, lim);
+    const int64_t nl = last ? el : (many ? first_near(lcol, kl, el, lim) : first_from(lcol, kl, el, lim));
+    const int64_t nu = last ? eu : (many ? first_near(col, ku, eu, lim) : first_from(col, ku, eu, lim));
     cnt[p * kMR + lr] = (uint16_t)(nl - kl + nu - ku);
     cntl[p * kMR + lr] = (uint16_t)(nl - kl);
     kl = nl;
@@ -537,33 +559,156 @@ __device__ __forceinline__ unsigned class_mask(unsigned in, unsigned b0, unsigne
   return in & ((c & 1) ? b0 : ~b0) & ((c & 2) ? b1 : ~b1) & ((c & 4) ? b2 : ~b2);
 }
 
-// CTA per panel, warp per stream, its 32 rows in turn: a first pass over the row's entries counts its
-// classes by ballots, a second one places every entry (the diagonal takes the row's last step: the
-// small off-diagonal terms are summed before the typically much larger diagonal one) in a shared-memory
-// row, padding included, which is written out in 16-byte pieces.  Reads are coalesced, every stream
-// position is written once.  A thread per row (segments read in column order, class sequence chosen
-// step by step, entries gathered in class order) took 8.3 ms for 3.0e8 entries; this takes 3.1.
-// Dynamic shared memory: per warp `cap` steps of columns and values (cap a multiple of 8, at least the
-// longest stream's).
-template <typename V>
-__global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
+// Rows of one stream that a warp places at a time: one, or four of at most kFewSteps steps.
+constexpr int kFewSteps = 64;
+// Panels of a row block from which on a row's first entry in a panel is searched for instead of summed up
+// from the counts of the panels before it.
+constexpr int kSumPanels = 32;
+
+// The streams' arrays, and the panel's tiles in shared memory.
+template <typename V> struct ScatterArgs {
+  const int32_t* lcol;
+  const V* lval;
+  const int32_t* col;
+  const V* val;
+  uint16_t* bcol;
+  V* bval;
+  const int32_t* s_tc;
+  const uint32_t* s_slot;
+  int nt, pr;
+};
+// Rows of one stream: lane l's row, its entries in the panel and those left of the diagonal, the first of
+// these and of the others.
+struct StreamRow {
+  int64_t r, el, eu;
+  int len, nl;
+};
+
+// Places the 32 rows of a stream of nblk blocks from blk0 on, LR lanes a row (32, or 8: four rows at a
+// time, which then have at most 8 * LR entries).  rv, rc: the warp's rows in shared memory, places: 8 each.
+template <typename V, int LR>
+__device__ __forceinline__ void scatter_rows(const ScatterArgs<V>& a, const StreamRow& mine, int64_t blk0, int nblk, V* rv0,
+                                             uint16_t* rc0, ClassPlace* places) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int E = BlkPiece<V>::kEpp;
+  const int lane = threadIdx.x & 31, sub = lane % LR, first = lane - sub, cls = lane & 7;
+  const unsigned group = LR == 32 ? kAll : ((1u << (LR & 31)) - 1u) << first, below = (1u << lane) - 1u;
+  ClassPlace* place_of = places + first / LR * 8;
+  V* rv = rv0 + first / LR * (nblk * kBS);
+  uint16_t* rc = rc0 + first / LR * (nblk * kBS);
+  for (int l0 = 0; l0 < 32; l0 += 32 / LR) {
+    const int l = l0 + first / LR;
+    const int64_t r = __shfl_sync(kAll, mine.r, l);
+    const int len = __shfl_sync(kAll, mine.len, l);
+    const int longest = LR == 32 ? len : __shfl_sync(kAll, mine.len, l0);   // rows are ranked by length
+    // entry q of the row: q < nl in the lower CSR, else in U
+    const int nl = __shfl_sync(kAll, mine.nl, l);
+    const int64_t el = __shfl_sync(kAll, mine.el, l), eu = __shfl_sync(kAll, mine.eu, l) - nl;
+    auto col_at = [&](int q) { return q < nl ? a.lcol[el + q] : a.col[eu + q]; };
+    auto val_at = [&](int q) { return q < nl ? a.lval[el + q] : a.val[eu + q]; };
+    // class counts of the off-diagonal entries (class cls of each lane), then their placement
+    int nc = 0, noff = 0, run = 0;
+    auto count = [&](int32_t c) {
+      const unsigned in = __ballot_sync(kAll, c >= 0 && (int64_t)c != r) & group;
+      const unsigned b0 = __ballot_sync(kAll, c & 1), b1 = __ballot_sync(kAll, c & 2);
+      const unsigned b2 = __ballot_sync(kAll, c & 4);
+      nc += __popc(class_mask(in, b0, b1, b2, cls));
+      noff += __popc(in);
+    };
+    auto place = [&](int32_t c, V v) {
+      const bool valid = c >= 0, offd = valid && (int64_t)c != r;
+      const unsigned in = __ballot_sync(kAll, offd) & group;
+      const unsigned b0 = __ballot_sync(kAll, c & 1), b1 = __ballot_sync(kAll, c & 2);
+      const unsigned b2 = __ballot_sync(kAll, c & 4);
+      const int cl = c & 7;
+      const int i = __shfl_sync(kAll, run, first + cl) + __popc(class_mask(in, b0, b1, b2, cl) & below);
+      run += __popc(class_mask(in, b0, b1, b2, cls));
+      if (valid) {
+        const int k = offd ? class_step(place_of[cl], cl, l, i) : len - 1;
+        const int32_t J = c / kMC;
+        const int lo = tile_index(a.s_slot, a.s_tc, a.nt, J);
+        rc[k] = (uint16_t)(lo * kMC + (c - J * kMC));
+        rv[k] = v;
+      }
+    };
+    auto set_places = [&]() {
+      const ClassPlace p = class_place(cls, nc, l, noff);
+      if (sub < 8) place_of[sub] = p;
+      __syncwarp();
+    };
+    if (longest <= 8 * LR) {
+      // read once, into registers, all loads in flight
+      int32_t c[8];
+      V v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const bool in = q * LR + sub < len;
+        c[q] = in ? col_at(q * LR + sub) : -1;
+        v[q] = V(0);
+        if (in) v[q] = val_at(q * LR + sub);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q * LR < longest) count(c[q]);
+      set_places();
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q * LR < longest) place(c[q], v[q]);
+    } else if (LR == 32) {
+      for (int q = lane; q - lane < len; q += 32) count(q < len ? col_at(q) : -1);
+      set_places();
+      for (int q = lane; q - lane < len; q += 32) {
+        V v = V(0);
+        if (q < len) v = val_at(q);
+        place(q < len ? col_at(q) : -1, v);
+      }
+    }
+    // padding: zero values on the zero row of the class the lane wants
+    for (int k = len + sub; k < nblk * kBS; k += LR) {
+      rc[k] = (uint16_t)(a.pr + ((l + k) & 7));
+      rv[k] = V(0);
+    }
+    __syncwarp();
+    for (int b = sub; b < nblk; b += LR) {
+      const int64_t at = (blk0 + b) * kBE;
+      *reinterpret_cast<uint4*>(a.bcol + at + l * kBS) = *reinterpret_cast<const uint4*>(rc + b * kBS);
+#pragma unroll
+      for (int u = 0; u < kBS; u += E)
+        *reinterpret_cast<uint4*>(a.bval + at + blk_value_at<V>(l, u)) = *reinterpret_cast<const uint4*>(rv + b * kBS + u);
+    }
+    __syncwarp();
+  }
+}
+
+// CTA per panel, warp per stream, its 32 rows in turn, or (FEW) four at a time where none has more than
+// kFewSteps entries: a first pass over a row's entries counts its classes by ballots, a second one places every
+// entry (the diagonal takes the row's last step: the small off-diagonal terms are summed before the
+// typically much larger diagonal one) in a shared-memory row, padding included, which is written out in
+// 16-byte pieces.  Reads are coalesced, every stream position is written once.  A thread per row (segments
+// read in column order, class sequence chosen step by step, entries gathered in class order) took 8.3 ms
+// for 3.0e8 entries; this takes 3.1.  Dynamic shared memory: per warp `cap` steps of columns and values
+// (a multiple of 8, at least scatter_cap of the longest stream).
+__host__ __device__ constexpr int scatter_cap(int steps) {
+  const int few = 4 * (steps < kFewSteps ? steps : kFewSteps);
+  return steps > few ? steps : few;
+}
+template <typename V, bool FEW>
+__global__ void __launch_bounds__(kMR, 4) k_rs_scatter(const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
                                                     const V* __restrict__ lval, const int64_t* __restrict__ rowptr,
                                                     const int32_t* __restrict__ col, const V* __restrict__ val, int64_t n,
                                                     const int32_t* __restrict__ rbp, const int32_t* __restrict__ pan_rb,
                                                     const int32_t* __restrict__ pt0, const int32_t* __restrict__ pnt,
                                                     const int32_t* __restrict__ tcol, const uint16_t* __restrict__ cnt,
-                                                    const uint16_t* __restrict__ cntl, const uint8_t* __restrict__ perm, const int64_t* __restrict__ sboff,
-                                                    int pr, int cap, uint16_t* __restrict__ bcol,
-                                                    V* __restrict__ bval) {
+                                                    const uint16_t* __restrict__ cntl, const uint8_t* __restrict__ perm,
+                                                    const int64_t* __restrict__ sboff, int pr, int cap,
+                                                    uint16_t* __restrict__ bcol, V* __restrict__ bval) {
   static_assert(kBS == 8 && (kBS * sizeof(V)) % 16 == 0 && kW == 8, "a lane's block is whole 16-byte pieces");
-  constexpr int E = BlkPiece<V>::kEpp;
   extern __shared__ __align__(16) unsigned char sm_rows[];
   __shared__ int32_t s_tc[32];
   __shared__ uint32_t s_slot[256];      // tile column J and its index in the panel, at J mod 256 (one of them)
-  __shared__ ClassPlace s_place[kW][8];
+  __shared__ ClassPlace s_place[kW][FEW ? 32 : 8];
   const int64_t p = blockIdx.x;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cls = lane & 7;
-  const unsigned below = (1u << lane) - 1u;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nt = pnt[p];
   if (threadIdx.x < 32) s_tc[threadIdx.x] = (int)threadIdx.x < nt ? tcol[pt0[p] + threadIdx.x] : INT32_MAX;
   s_slot[threadIdx.x] = 0xffffffffu;
@@ -574,102 +719,35 @@ __global__ void __launch_bounds__(kMR) k_rs_scatter(const int64_t* __restrict__ 
   uint16_t* rc = reinterpret_cast<uint16_t*>(reinterpret_cast<V*>(sm_rows) + (size_t)kW * cap) + (size_t)w * cap;
   const int64_t I = pan_rb[p], blk0 = sboff[p * kW + w];
   const int nblk = (int)(sboff[p * kW + w + 1] - blk0);
-  const int p_first = rbp[I];
-  // lane l: row of the stream's lane l, its entries in the panel
+  if (nblk == 0) return;
+  const int64_t p_first = rbp[I];
   const int my_lr = perm[p * kMR + w * 32 + lane];
-  int my_len = 0, my_nl = 0;       // of which left of the diagonal
-  int64_t my_el = 0, my_eu = 0;    // first of those, first of the others
-  if (I * kMR + my_lr < n) {
-    my_len = cnt[p * kMR + my_lr];
-    my_nl = cntl[p * kMR + my_lr];
-    my_el = lptr[I * kMR + my_lr];
-    my_eu = rowptr[I * kMR + my_lr];
-    for (int64_t q = p_first; q < p; ++q) {
-      const int nl = cntl[q * kMR + my_lr];
-      my_el += nl;
-      my_eu += cnt[q * kMR + my_lr] - nl;
-    }
-  }
-  for (int l = 0; l < 32; ++l) {
-    const int64_t r = I * kMR + __shfl_sync(0xffffffffu, my_lr, l);
-    const int len = __shfl_sync(0xffffffffu, my_len, l);
-    // entry q of the row: q < nl in the lower CSR, else in U
-    const int nl = __shfl_sync(0xffffffffu, my_nl, l);
-    const int64_t el = __shfl_sync(0xffffffffu, my_el, l), eu = __shfl_sync(0xffffffffu, my_eu, l) - nl;
-    auto col_at = [&](int q) { return q < nl ? lcol[el + q] : col[eu + q]; };
-    auto val_at = [&](int q) { return q < nl ? lval[el + q] : val[eu + q]; };
-    // class counts of the off-diagonal entries (class cls of each lane), then their placement
-    int nc = 0, noff = 0, run = 0;
-    auto count = [&](int32_t c) {
-      const unsigned in = __ballot_sync(0xffffffffu, c >= 0 && (int64_t)c != r);
-      const unsigned b0 = __ballot_sync(0xffffffffu, c & 1), b1 = __ballot_sync(0xffffffffu, c & 2);
-      const unsigned b2 = __ballot_sync(0xffffffffu, c & 4);
-      nc += __popc(class_mask(in, b0, b1, b2, cls));
-      noff += __popc(in);
-    };
-    auto place = [&](int32_t c, V v) {
-      const bool valid = c >= 0, offd = valid && (int64_t)c != r;
-      const unsigned in = __ballot_sync(0xffffffffu, offd);
-      const unsigned b0 = __ballot_sync(0xffffffffu, c & 1), b1 = __ballot_sync(0xffffffffu, c & 2);
-      const unsigned b2 = __ballot_sync(0xffffffffu, c & 4);
-      const int cl = c & 7;
-      const int i = __shfl_sync(0xffffffffu, run, cl) + __popc(class_mask(in, b0, b1, b2, cl) & below);
-      run += __popc(class_mask(in, b0, b1, b2, cls));
-      if (valid) {
-        const int k = offd ? class_step(s_place[w][cl], cl, l, i) : len - 1;
-        const int32_t J = c / kMC;
-        const int lo = tile_index(s_slot, s_tc, nt, J);
-        rc[k] = (uint16_t)(lo * kMC + (c - J * kMC));
-        rv[k] = v;
+  StreamRow mine = {I * kMR + my_lr, 0, 0, 0, 0};
+  if (mine.r < n) {
+    mine.len = cnt[p * kMR + my_lr];
+    mine.nl = cntl[p * kMR + my_lr];
+    mine.el = lptr[mine.r];
+    mine.eu = rowptr[mine.r];
+    if (p - p_first <= kSumPanels) {
+      for (int64_t q = p_first; q < p; ++q) {
+        const int nl = cntl[q * kMR + my_lr];
+        mine.el += nl;
+        mine.eu += cnt[q * kMR + my_lr] - nl;
       }
-    };
-    auto set_places = [&]() {
-      const ClassPlace mine = class_place(cls, nc, l, noff);
-      if (lane < 8) s_place[w][lane] = mine;
-      __syncwarp();
-    };
-    if (len <= 256) {
-      // read once, into registers, all loads in flight
-      int32_t c[8];
-      V v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const bool in = q * 32 + lane < len;
-        c[q] = in ? col_at(q * 32 + lane) : -1;
-        v[q] = V(0);
-        if (in) v[q] = val_at(q * 32 + lane);
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q * 32 < len) count(c[q]);
-      set_places();
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q * 32 < len) place(c[q], v[q]);
     } else {
-      for (int q = lane; q - lane < len; q += 32) count(q < len ? col_at(q) : -1);
-      set_places();
-      for (int q = lane; q - lane < len; q += 32) {
-        V v = V(0);
-        if (q < len) v = val_at(q);
-        place(q < len ? col_at(q) : -1, v);
-      }
+      const int64_t lim = (panel_last_cb(pt0, pnt, tcol, p - 1) + 1) * kMC;
+      mine.el = first_from(lcol, mine.el, lptr[mine.r + 1], lim);
+      mine.eu = first_from(col, mine.eu, rowptr[mine.r + 1], lim);
     }
-    // padding: zero values on the zero row of the class the lane wants
-    for (int k = len + lane; k < nblk * kBS; k += 32) {
-      rc[k] = (uint16_t)(pr + ((l + k) & 7));
-      rv[k] = V(0);
-    }
-    __syncwarp();
-    for (int b = lane; b < nblk; b += 32) {
-      const int64_t at = (blk0 + b) * kBE;
-      *reinterpret_cast<uint4*>(bcol + at + l * kBS) = *reinterpret_cast<const uint4*>(rc + b * kBS);
-#pragma unroll
-      for (int u = 0; u < kBS; u += E)
-        *reinterpret_cast<uint4*>(bval + at + blk_value_at<V>(l, u)) = *reinterpret_cast<const uint4*>(rv + b * kBS + u);
-    }
-    __syncwarp();
   }
+  const ScatterArgs<V> a = {lcol, lval, col, val, bcol, bval, s_tc, s_slot, nt, pr};
+  if constexpr (FEW) {
+    if (nblk * kBS <= kFewSteps) {
+      scatter_rows<V, 8>(a, mine, blk0, nblk, rv, rc, s_place[w]);
+      return;
+    }
+  }
+  scatter_rows<V, 32>(a, mine, blk0, nblk, rv, rc, s_place[w]);
 }
 
 // Row groups of a row block.  With fewer row blocks than SMs each half of a row block is a CTA of
@@ -928,10 +1006,20 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
   const int64_t nent = std::max<int64_t>(nblk, 1) * kBE;
   EIG_TRY(reserve_streams(P, nent, sizeof(V)));
   if (nblk > 0) {
-    const int cap = (*std::max_element(h_steps.begin(), h_steps.end()) + kBS - 1) / kBS * kBS;
+    // four rows at a time where half of the streams that have entries at all are short (without that path the
+    // kernel is a fiftieth faster)
+    int64_t some = 0, few = 0;
+    for (int32_t x : h_steps) {
+      some += x > 0;
+      few += x > 0 && x <= kFewSteps;
+    }
+    const bool by_four = 2 * few >= some;
+    const int steps = (*std::max_element(h_steps.begin(), h_steps.end()) + kBS - 1) / kBS * kBS;
+    const int cap = by_four ? scatter_cap(steps) : steps;
     const size_t sm = (size_t)kW * cap * (2 + sizeof(V));
-    if (sm > 40 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(k_rs_scatter<V>, sm));
-    k_rs_scatter<V><<<(unsigned)npan, kMR, sm, st>>>(
+    auto scatter = by_four ? k_rs_scatter<V, true> : k_rs_scatter<V, false>;
+    if (sm > 40 * 1024) EIG_CUDA_TRY(::eig::ensure_dyn_smem(scatter, sm));
+    scatter<<<(unsigned)npan, kMR, sm, st>>>(
         lptr.as<int64_t>(), lcol.as<int32_t>(), lval.as<V>(), P->rowptr, P->col, val, n, P->m_rbp.as<int32_t>(),
         d_pan_rb.as<int32_t>(), P->m_pt0.as<int32_t>(), P->m_pnt.as<int32_t>(), P->m_tcol.as<int32_t>(),
         cntp.as<uint16_t>(), cntl.as<uint16_t>(), P->m_perm.as<uint8_t>(), P->m_sboff.as<int64_t>(), P->m_pr, cap,
