@@ -55,11 +55,12 @@ eig_status eig_gram_noalloc_parts(const void* A, const void* B, int64_t n, int n
   if (max_parts < 1 || max_parts > kNoAllocParts) return EIG_EINVAL;
   void* scratch = nullptr;
   EIG_TRY(scratch_address(&scratch));
+  // as eig_gram has it, so that the sums are grouped the same
   BlockList bl;
-  bl.n = 2;
+  bl.n = A == B ? 1 : 2;
   bl.p[0] = A;
   bl.p[1] = B;
-  const int pa = 0, pb = 1;
+  const int pa = 0, pb = bl.n - 1;
   // every CTA overwrites all of its partials, so the array needs no clearing between calls
   return gram_multi(bl, &pa, &pb, 1, nb, n, vec_type, G, scratch, as_stream(stream), max_parts);
 }

@@ -66,3 +66,17 @@ def test_gram_noalloc_parts_rejects_bad_cap():
         with pytest.raises(binding.EigError) as e:
             binding.gram_noalloc(A, A, max_parts=bad)
         assert e.value.status == binding.EIG_EINVAL
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n,nb", [(33, 8), (70001, 5), (200003, 16), (400000, 8), (100003, 32)])
+@pytest.mark.parametrize("same", [False, True])
+def test_gram_noalloc_equals_gram_bitwise(dt, n, nb, same):
+    """The partials of eig_gram fit the fixed array, so both calls must group and round alike, also for a
+    block with itself (of which eig_gram multiplies the upper tiles only)."""
+    from paper_2305_15552_gb300 import binding
+    binding.load()
+    rng = np.random.default_rng(n + nb)
+    A = torch.tensor(rng.standard_normal((n, nb)), dtype=dt, device="cuda")
+    B = A if same else torch.tensor(rng.standard_normal((n, nb)), dtype=dt, device="cuda")
+    assert torch.equal(binding.gram_noalloc(A, B), binding.gram(A, B))
