@@ -80,3 +80,26 @@ def test_gram_noalloc_equals_gram_bitwise(dt, n, nb, same):
     A = torch.tensor(rng.standard_normal((n, nb)), dtype=dt, device="cuda")
     B = A if same else torch.tensor(rng.standard_normal((n, nb)), dtype=dt, device="cuda")
     assert torch.equal(binding.gram_noalloc(A, B), binding.gram(A, B))
+
+
+@pytest.mark.parametrize("nb", [8, 16, 32])
+def test_gram_totals_over_many_chunks(nb):
+    """FP32 chunk sums (32 rows) into one partial: a block whose chunks hold one nonzero product each, 1
+    in the first chunks (of every group of threads that may share the rows) and a constant far below
+    it in the others.  Every chunk sum is exact, so the total may lose 2^-48 of itself per chunk (double
+    that for both roundings of the pair), and the partials' FP64 sum a few 2^-53."""
+    from paper_2305_15552_gb300 import binding
+    binding.load()
+    chunks, first = 65536, 32
+    c = np.float32(5.603129e-08) * np.float32(2.0) ** -np.arange(nb, dtype=np.float32)
+    a = np.zeros((chunks, 32, nb), np.float32)
+    a[:first, 0] = 1.0
+    a[first:, 0] = c
+    A = torch.tensor(a.reshape(-1, nb), device="cuda")
+    ones = torch.ones_like(A)
+    want = first + (chunks - first) * c.astype(np.float64)
+    for x, y in ((A, ones), (ones, A)):
+        for parts in (1, 3):
+            got = binding.gram_noalloc(x, y, max_parts=parts).cpu().numpy()
+            got = got if x is A else got.T
+            assert np.all(np.abs(got - want[:, None]) <= chunks * 2.0 ** -47 * want[:, None])
