@@ -349,3 +349,23 @@ def test_plan_memory_of_scattered_entries():
     finally:
         del rest
         torch.cuda.empty_cache()
+
+
+# more tiles than threads, so that a thread takes two (17, 34; 62 with itself) or four (31, 62) of them and
+# one group takes the chunk: odd widths with 1 x 1 tiles, widths of 2 mod 4 with 2 x 2
+@pytest.mark.parametrize("n", [31, 304 * 32 * 2 + 45])
+@pytest.mark.parametrize("nb", [17, 31, 34, 62])
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_gram_several_tiles_a_thread(n, nb, dt):
+    from paper_2305_15552_gb300 import binding as B
+    rng = np.random.default_rng(n + nb)
+    a, b = rng.standard_normal((n, nb)), rng.standard_normal((n, nb))
+    A, Bm = torch.tensor(a, dtype=dt, device="cuda"), torch.tensor(b, dtype=dt, device="cuda")
+    for X, Y in ((A, Bm), (A, A), (_shifted(a, dt), Bm)):
+        G = B.gram(X, Y).cpu().numpy()
+        Xe, Ye = X.double().cpu().numpy(), Y.double().cpu().numpy()
+        # as in test_gram_chunk_edges
+        tol = (2.0 ** -24 * 40 if dt == torch.float32 else 2.0 ** -53 * (n + 10)) * (np.abs(Xe).T @ np.abs(Ye)) + 1e-300
+        assert np.all(np.abs(G - Xe.T @ Ye) <= tol)
+        if X is Y:
+            assert np.array_equal(G, G.T)
