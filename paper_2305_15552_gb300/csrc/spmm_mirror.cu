@@ -945,9 +945,9 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
   P->m_pr = std::max(1, *std::max_element(pnt.begin(), pnt.end())) * kMC;
   P->m_groups = row_groups(nRB);
   at = 0;
-  EIG_TRY(P->m_own.reserve(DevBuf::part(nRB * 4) + DevBuf::part((nRB + 1) * 4) + 2 * DevBuf::part(npan * 4) + DevBuf::part(npan * kMR) +
+  EIG_TRY(P->m_own.reserve(DevBuf::part(nRB * 16) + DevBuf::part((nRB + 1) * 4) + 2 * DevBuf::part(npan * 4) + DevBuf::part(npan * kMR) +
                            DevBuf::part(npan * kW * 4) + DevBuf::part((npan * kW + 1) * 8)));
-  P->m_order.borrow(P->m_own, nRB * 4, &at);
+  P->m_order.borrow(P->m_own, nRB * 16, &at);
   P->m_rbp.borrow(P->m_own, (nRB + 1) * 4, &at);
   P->m_pt0.borrow(P->m_own, npan * 4, &at);
   P->m_pnt.borrow(P->m_own, npan * 4, &at);
@@ -987,7 +987,8 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
   // Row blocks in order of work, the longest first (a counting sort, stable): CTAs are started in this
   // order, so that the last ones to run are short.  In index order / in this order, us: n = 197,822 with
   // 1080 nonzeros a row, FP32, nb 16: 573 / 499, nb 8: 358 / 290; n = 663,527 with 300, FP64 vectors, nb 8:
-  // 830 / 730; n = 2M with 400, FP32, nb 16: 1750 / 1709.
+  // 830 / 730; n = 2M with 400, FP32, nb 16: 1750 / 1709.  A row block's panels stand beside its number, so
+  // that a CTA starts with one load and not two in a row.
   {
     std::vector<int64_t> work(nRB);
     int64_t longest = 0;
@@ -998,9 +999,9 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
     std::vector<int64_t> start(longest + 2, 0);
     for (int64_t x : work) start[longest - x + 1]++;
     for (int64_t l = 0; l <= longest; ++l) start[l + 1] += start[l];
-    std::vector<int32_t> order(nRB);
-    for (int64_t I = 0; I < nRB; ++I) order[start[longest - work[I]]++] = (int32_t)I;
-    EIG_CUDA_TRY(cudaMemcpyAsync(P->m_order.p, order.data(), nRB * 4, cudaMemcpyHostToDevice, st));
+    std::vector<int4> order(nRB);
+    for (int64_t I = 0; I < nRB; ++I) order[start[longest - work[I]]++] = make_int4((int)I, rbp[I], rbp[I + 1], 0);
+    EIG_CUDA_TRY(cudaMemcpyAsync(P->m_order.p, order.data(), nRB * 16, cudaMemcpyHostToDevice, st));
   }
   // 5. the streams
   const int64_t nent = std::max<int64_t>(nblk, 1) * kBE;
@@ -1035,8 +1036,7 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
 // ---------------------------------------------------------------------------------------
 struct RsArgs {
   int64_t n;
-  const int32_t* order;
-  const int32_t* rbp;
+  const int4* order;
   const int32_t* pt0;
   const int32_t* pnt;
   const int32_t* tcol;
@@ -1337,9 +1337,9 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
   // warps of a scheduler (every fourth) take a long and a short stream: 0 1 2 3 7 6 5 4
   const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
   const int w = w0 + (wi < 4 ? wi : 11 - wi);
-  const int64_t I = a.order[slot];
-  const int64_t r0 = I * kMR;
-  const int p0 = a.rbp[I], p1 = a.rbp[I + 1];
+  const int4 blk = a.order[slot];
+  const int64_t r0 = (int64_t)blk.x * kMR;
+  const int p0 = blk.y, p1 = blk.z;
 
   // zero rows (one per class) for the padding entries; never overwritten by staging
   for (int i = tid; i < 8 * RBY / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(xs + (size_t)a.pr * RBY)[i] = 0u;
@@ -1740,8 +1740,7 @@ template <typename T, typename V> struct RsSlice<T, V, 1> { static constexpr int
 static RsArgs rs_args(SpmmPlan* P) {
   RsArgs a;
   a.n = P->n;
-  a.order = P->m_order.as<int32_t>();
-  a.rbp = P->m_rbp.as<int32_t>();
+  a.order = P->m_order.as<int4>();
   a.pt0 = P->m_pt0.as<int32_t>();
   a.pnt = P->m_pnt.as<int32_t>();
   a.tcol = P->m_tcol.as<int32_t>();
