@@ -275,6 +275,7 @@ eig_status spmm_plan_build(SpmmPlan* P, const eig_csr_upper* H, int R, int C, in
     P->layout = EIG_LAYOUT_MIRRORED;
     return EIG_OK;
   }
+  tmp.mem.release();   // the bitmap alone is n^2 / 131,072 bytes
   std::vector<int32_t> h_sched_cb;
   std::vector<int64_t> h_sched_ptr(1, 0);
   for (int64_t J = 0; J < P->nCB; ++J) {

@@ -369,3 +369,41 @@ def test_gram_several_tiles_a_thread(n, nb, dt):
         assert np.all(np.abs(G - Xe.T @ Ye) <= tol)
         if X is Y:
             assert np.array_equal(G, G.T)
+
+
+def test_plan_memory_of_half_layout():
+    """16M rows: the tile bitmap (2.0 GB) is gone before the half-stored copy (0.6 GB) is built, so that
+    2.4 GB are enough for the plan."""
+    from gen.synth import CSRUpper
+    from paper_2305_15552_gb300 import binding as B
+    n = 16_000_000
+    # the diagonal (2) and, for every row but the last 64, the column 64 to the right (1)
+    rowptr = np.minimum(2 * np.arange(n + 1, dtype=np.int64), np.arange(n + 1, dtype=np.int64) + n - 64)
+    i = np.arange(n, dtype=np.int64)
+    col = np.empty(rowptr[-1], np.int32)
+    val = np.full(rowptr[-1], 2.0)
+    col[rowptr[:-1]] = i
+    col[rowptr[:n - 64] + 1] = i[:n - 64] + 64
+    val[rowptr[:n - 64] + 1] = 1.0
+    H = CSRUpper(n=n, rowptr=rowptr, col=col, val=val, storage="f64")
+    dev = tuple(torch.tensor(x, device="cuda") for x in (H.rowptr, H.col, H.val))
+    x = torch.tensor(np.arange(n) % 7, dtype=torch.float64, device="cuda").reshape(n, 1)
+    y = torch.empty_like(x)
+    small = CSRUpper(n=64, rowptr=np.arange(65), col=np.arange(64, dtype=np.int32), val=np.ones(64), storage="f64")
+    B.SpmmPlan(small, layout="half").close()      # code loaded
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - 2_400_000_000, dtype=torch.uint8, device="cuda")
+    try:
+        P = B.SpmmPlan(H, device_arrays=dev, layout="half", copy=False)
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    assert P.info()["layout"] == B.LAYOUTS["half"]
+    P.spmm(x, y)
+    P.close()
+    v = np.arange(n) % 7
+    want = 2.0 * v
+    want[:-64] += v[64:]
+    want[64:] += v[:-64]
+    assert np.array_equal(y.cpu().numpy()[:, 0], want)
