@@ -262,6 +262,11 @@ __global__ void k_reduce_partials(const double* __restrict__ part, int nparts, i
 
 // Two CTAs per SM, each with a near-equal share of the rows in units of 32 rows (the FP32 chunks) or
 // 8 (FP64, bound by its pipe: 20,000 rows are 66 per CTA instead of 96 in 209 of them).
+// The grid also fixes how the rows are grouped into partial sums, and so the rounding of every Gram, to
+// which the last iterations of the hybrid solve are sensitive: at n = 2M (tolerance 1e-6, 4 + 5 iterations)
+// its largest residual is 9.8e-7 with two CTAs per SM, 9.9e-7 with one and a half, 6.7e-7 with one, and was
+// 6.9e-7 with shares of equal whole chunks; another start took 7 RMM-DIIS iterations with two CTAs per SM
+// and 21 with four.
 static int gram_grid(int64_t n, eig_dtype vt, int64_t* units, int max_parts) {
   const int unit = vt == EIG_F32 ? kGramRows : 8;
   int64_t g = num_sms() * 2;
@@ -329,8 +334,11 @@ eig_status gram_multi(const BlockList& blocks, const int* pa, const int* pb, int
   const int TM = (nb % 4 == 0) ? 4 : ((nb % 2 == 0) ? 2 : 1);
   if ((size_t)npairs * (nb / TM) * (nb / TM) > 4 * kGramThreads) return EIG_EUNSUPPORTED;
   if (vt == EIG_F32) {
-    // from 128 tiles of 4 x 4 on (LOBPCG's twelve pairs at nb = 16 have 174) the shared-memory pipe
-    // is the bound, and 8 x 4 tiles need two thirds of its loads; at most one tile a thread
+    // From 128 tiles of 4 x 4 on (of all pairs, a pair of a block with itself counted whole), 8 x 4 tiles:
+    // two thirds of the loads from shared memory, but half the threads.  Set at LOBPCG's twelve pairs,
+    // nb = 16, n = 2M (174 tiles): 416 us, 480 with 4 x 4.  One pair, n = 500,000, us with 4 x 4 / 8 x 4 tiles:
+    // nb = 40 (below the line) 93 / 93, 48 136 / 124, 56 159 / 163, 64 163 / 166; a block with itself: 40 60 / 69,
+    // 48 75 / 86, 56 97 / 102, 64 136 / 124.  n = 20,000: 48 30 / 39, 64 34 / 44: single pairs hardly gain.
     const int t8 = npairs * (nb / 8) * (nb / 4);
     if (nb % 8 == 0 && 2 * t8 > 128 && t8 <= kGramThreads)
       return gram_launch<float, 8, 4>(blocks, pl, nb, n, G, part, st, max_parts);

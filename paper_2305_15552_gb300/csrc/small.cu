@@ -228,9 +228,10 @@ __device__ __forceinline__ int sturm_count(const R* __restrict__ d, const R* __r
   R pm = 1.0, pc = d[0] - x;
   if (lead_f32(pc) == 0.0f) pc = R(-0x1p-40);
   int c = sign_bit(pc);
-  // What bounds it: the recurrence's dependent operations.  The next step's shifted diagonal and e2 are loaded and formed ahead of it, and the rescale is a
-  // multiplication by 1 or 2^+-64 instead of branches (a step at two warps per scheduler: 203 -> 160 cycles;
-  // four warps issue ~68 instructions each and take 255, 273 before).
+  // What bounds it: the recurrence's dependent operations.  The next step's shifted diagonal and e2 are
+  // loaded and formed ahead of it, and the rescale is a multiplication by 1 or 2^+-64 instead of
+  // branches (a step at two warps per scheduler: 203 -> 160 cycles; four warps issue ~68 instructions
+  // each and take 255, 273 before).
   R dn = (k > 1) ? d[1] - x : R(0.0), en = (k > 1) ? e2[0] : R(0.0);
   for (int i = 1; i < k; ++i) {
     const R dx = dn, t = en * pm;

@@ -63,7 +63,7 @@ struct SpmmPlan {
   DevBuf m_own, m_streams;           // the panel arrays; m_bcol and m_bval
   int64_t m_npan = 0, m_nblk = 0;
   int m_pr = 0, m_groups = 1;        // staged X rows of the widest panel; row groups (CTAs) per row block
-  DevBuf m_order;                    // int4[nRB]: row blocks (number, first panel, last + 1) by falling number of streamed blocks
+  DevBuf m_order;                    // int4[nRB]: row block, its first panel, its last + 1; most streamed blocks first
   DevBuf m_rbp;                      // int32[nRB+1]: panels of row block I
   DevBuf m_pt0, m_pnt;               // int32[m_npan]: first tile (into m_tcol) and tile count
   DevBuf m_tcol;                     // int32: column block of each tile of the mirrored matrix

@@ -516,14 +516,14 @@ __device__ __forceinline__ int64_t blk_value_at(int lane, int step) {
 // the row has entries of it get one (the last ones take the other parity's surplus: the only steps that
 // cost a conflict at nb >= 16 in FP32); of those that want a class mod 4 the same within the parity, of
 // those that want a class mod 8 within the class mod 4.
-// Step of entry i (columns ascending) of class c:
-struct ClassPlace {
+// Step of entry i (columns ascending) of class c (16-byte aligned: two loads a place):
+struct alignas(16) ClassPlace {
   int own;            // i < own: the i-th step that wants c
   int in8, base8;     // the next in8: steps that want c ^ 4, from its base8-th on
   int skip, in4;      // then the surplus of the class mod 4 (the c with bit 2 after the other one): its first
   int base4;          // in4 in steps that want (c ^ 2) mod 4, from the base4-th on,
   int base2;          // the rest in steps of the other parity, from the base2-th on
-  int pad;
+  int to_32_bytes;
 };
 __device__ __forceinline__ int half_from(int m, int first) { return m > first ? (m - first + 1) >> 1 : 0; }
 __device__ __forceinline__ int class_step(const ClassPlace& g, int c, int l, int i) {
@@ -753,7 +753,9 @@ __global__ void __launch_bounds__(kMR, 4) k_rs_scatter(const int64_t* __restrict
 // Row groups of a row block.  With fewer row blocks than SMs each half of a row block is a CTA of
 // its own: ranking within a half pads one to two percent more and X is staged twice, but n = 20,000
 // (79 row blocks, 100 nonzeros a row, FP32) takes 22.7 instead of 28.2 us at nb = 8 and 25.5 instead
-// of 32.8 at nb = 16; at 196 row blocks it no longer gains, at 391 it loses.
+// of 32.8 at nb = 16; at 196 row blocks it no longer gains, at 391 it loses.  At nb = 32, where one CTA's X
+// fills an SM, it gains with long rows (300 a row 101 -> 71) and loses a little with short ones (n = 36,000,
+// 140 a row: 58 -> 63).
 int row_groups(int64_t nRB) { return nRB < num_sms() ? 2 : 1; }
 
 // ---------------------------------------------------------------------------------------
@@ -762,9 +764,11 @@ int row_groups(int64_t nRB) { return nRB < num_sms() ? 2 : 1; }
 // FP64 products run at the FP64 pipe's rate (one warp multiply-add per 64 clocks per scheduler), so
 // what matters is that every scheduler has the same number of them; with few rows, row blocks of
 // unequal length on unequal numbers of CTAs per SM left the busiest scheduler with 2.6 times the
-// average (n = 20,000, 100 nonzeros a row).  The columns are row indices of X in 16 bits, hence the
-// bound on n; there (65,000 rows, 100 or 400 nonzeros a row) the direct streams still take 0.56 and
-// 0.57 of the panels' time at nb = 8 (100 against 177 us, 385 against 677) and 0.51 to 0.57 at nb = 1.
+// average (n = 20,000, 100 nonzeros a row).  The bound on n is that of the streams' 16-bit columns, which
+// are row indices of X here, and not where the panels catch up: at 65,000 rows with 100 or 400 nonzeros a
+// row the direct streams take 0.60 and 0.66 of the panels' time at nb = 8 (105 against 175 us, 369
+// against 563) and 0.54 and 0.56 at nb = 1 (23 against 42, 65 against 116), so a product of 65,536 rows
+// takes that much longer than one of 65,535.
 bool direct_plan(const SpmmPlan* P) { return P->val_type == EIG_F64 && P->n < 65536; }
 
 // Warp per row: its entries, columns ascending and the diagonal last, dealt to its `split` lanes in
@@ -1375,7 +1379,8 @@ __device__ __forceinline__ void mirror_row_block(const RsArgs& a, const T* __res
     } else if (DF && NB >= 2 && ld == NB) {
       if constexpr (DF && NB >= 2) stage_df_rows<NB>(xs, X, a.tcol + t0, npt, a.n);
     } else {
-      // a whole CTA (the host does not split row blocks here): a constant stride
+      // a whole CTA (the host does not split row blocks here): a constant stride, with which the divisions
+      // below fold (FP64 values, nb = 32, scattered entries, n = 200,000: 29.5 ms, 63.9 with blockDim.x)
       for (int64_t i = tid; i < (int64_t)npt * kMC * NB; i += kW * 32) {
         const int t = (int)(i / (kMC * NB));
         const int rr = (int)((i / NB) % kMC), e = (int)(i % NB);
@@ -1546,7 +1551,7 @@ k_spmm_mirror_batch(const __grid_constant__ MirrorBatch B) {
 // average) is not the makespan; the launch order pairs long with short ones on an SM: CTAs (four warps,
 // one per scheduler, of near-equal length) come in order of length, and every second round of one CTA
 // per SM in the reverse order.  n = 20,000, 100 nonzeros a row: 41 us at nb = 8 (27 us of FP64
-// multiply-adds), 76 at nb = 16, 12.5 at nb = 1; with row blocks and panels 143, 262 and 38.
+// multiply-adds), 76 at nb = 16, 14 at nb = 1; with row blocks and panels 108, 195 and 34.
 struct DirectArgs {
   int64_t n;
   int32_t nw;            // warps' worth of slots
@@ -1568,7 +1573,8 @@ __device__ __forceinline__ Vec<double, 4> ld_sector(const double* p) {
 }
 
 // SECTOR (NB = 4): every gathered piece starts on a 32-byte boundary.  The products' inputs are only
-// aligned to 16 bytes, and a 32-byte load from such an address faults, so the host looks at X.
+// aligned to 16 bytes, and a 32-byte load from such an address faults, so the host looks at X.  Two 16-byte
+// loads cost little (n = 20,000, 100 nonzeros a row, X aligned / off by 16 bytes: nb = 8 43 / 44 us, 16 76 / 79).
 template <int NB, bool CHEB, bool SECTOR>
 __global__ void __launch_bounds__(kDirectWarps * 32, 4)
 k_spmm_direct(const __grid_constant__ DirectArgs a, const double* __restrict__ X, double* __restrict__ Y, int ld,
