@@ -589,8 +589,8 @@ SHAPE_NAMES = {0: "FP32 vectors, nb 1", 1: "FP32 vectors, nb 2", 2: "FP32 vector
 # DRAM bytes per layout entry of k_spmm_mirror, from one ncu capture per shape at n = 500,000
 # (dram__bytes_read.sum + dram__bytes_write.sum over the plan's layout entries, 2.04e8); keyed
 # by the shape index 6 * (FP64 vectors) + log2(nb); void once spmm_mirror.cu changes.
-SPMM_TRAFFIC = {"kernel_sha": "d9766173fd92e677", "per_layout_entry": {4: 1.311984e9 / 204360448, 3: 1.264898e9 / 204360448,
-                                                          9: 1.335628e9 / 204360448}}
+SPMM_TRAFFIC = {"kernel_sha": "2bd61e47e79eb4dd", "per_layout_entry": {4: 1.314712e9 / 204360448, 3: 1.266262e9 / 204360448,
+                                                          9: 1.335377e9 / 204360448}}
 
 
 def kernel_sha():

@@ -1,6 +1,8 @@
 // Tall-skinny dense kernels: Gram products (Eq. rreig's S^T S and S^T H S; Eq. bgs's V^T W),
 // block-times-small-matrix products (Eqs. xupd, pupd; CholQR's X R^{-1}), the fused LOBPCG
 // update, and deterministic reductions.  All are HBM-bound passes over n x nb blocks.
+#include <type_traits>
+
 #include "common.cuh"
 #include "dense.cuh"
 #include "vec.cuh"
@@ -119,8 +121,8 @@ __host__ __device__ inline bool gram_tile(const PairList& pairs, int nb, int idx
 // What bounds it: one pair is an HBM pass; many pairs the shared-memory pipe (a 4 x 4 tile takes
 // six clocks of loads for four clocks of multiply-adds per row, an 8 x 4 tile eight for eight), FP64
 // the FP64 pipe (two lanes per clock per SM: hence only the upper tiles of a pair of a block with
-// itself).  Measured: one FP32 pair at n = 2M, nb = 16 in 57 us (4.5 TB/s; 204 us when one group of 16
-// threads multiplied), LOBPCG's twelve pairs there 416 us (480 us with 4 x 4 tiles); twelve FP64 pairs at
+// itself).  Measured: one FP32 pair at n = 2M, nb = 16 in 53 us (4.8 TB/s; 204 us when one group of 16
+// threads multiplied), LOBPCG's twelve pairs there 441 us (515 us with 4 x 4 tiles); twelve FP64 pairs at
 // n = 20,000, nb = 8 in 40 us (56 us).
 template <typename T, int TMI, int TMJ, int MAXT, bool PIPE>
 __global__ void __launch_bounds__(kGramThreads)
@@ -336,7 +338,7 @@ eig_status gram_multi(const BlockList& blocks, const int* pa, const int* pb, int
   if (vt == EIG_F32) {
     // From 128 tiles of 4 x 4 on (of all pairs, a pair of a block with itself counted whole), 8 x 4 tiles:
     // two thirds of the loads from shared memory, but half the threads.  Set at LOBPCG's twelve pairs,
-    // nb = 16, n = 2M (174 tiles): 416 us, 480 with 4 x 4.  One pair, n = 500,000, us with 4 x 4 / 8 x 4 tiles:
+    // nb = 16, n = 2M (174 tiles): 441 us, 515 with 4 x 4.  One pair, n = 500,000, us with 4 x 4 / 8 x 4 tiles:
     // nb = 40 (below the line) 93 / 93, 48 136 / 124, 56 159 / 163, 64 163 / 166; a block with itself: 40 60 / 69,
     // 48 75 / 86, 56 97 / 102, 64 136 / 124.  n = 20,000: 48 30 / 39, 64 34 / 44: single pairs hardly gain.
     const int t8 = npairs * (nb / 8) * (nb / 4);
@@ -425,10 +427,14 @@ eig_status rows_apply(const void* In, int nb, const double* M, void* Out, int64_
     return EIG_EUNSUPPORTED;
   const int rows = 8 * 4 * (32 / (nb * (vt == EIG_F64 ? 8 : 4) / 16));   // rows of one CTA pass
   const int grid = (int)max64(1, min64((n + rows - 1) / rows, (int64_t)num_sms() * 4));
-  if (vt == EIG_F32 && nb == 8) k_rows_apply<float, 8><<<grid, 256, 0, st>>>((const float*)In, M, (float*)Out, n, skip);
-  else if (vt == EIG_F32) k_rows_apply<float, 16><<<grid, 256, 0, st>>>((const float*)In, M, (float*)Out, n, skip);
-  else if (vt == EIG_F64 && nb == 8) k_rows_apply<double, 8><<<grid, 256, 0, st>>>((const double*)In, M, (double*)Out, n, skip);
-  else if (vt == EIG_F64) k_rows_apply<double, 16><<<grid, 256, 0, st>>>((const double*)In, M, (double*)Out, n, skip);
+  auto go = [&](auto kern, auto* out) {
+    typedef std::remove_pointer_t<decltype(out)> T;
+    kern<<<grid, 256, 0, st>>>(static_cast<const T*>(In), M, out, n, skip);
+  };
+  if (vt == EIG_F32 && nb == 8) go(k_rows_apply<float, 8>, static_cast<float*>(Out));
+  else if (vt == EIG_F32) go(k_rows_apply<float, 16>, static_cast<float*>(Out));
+  else if (vt == EIG_F64 && nb == 8) go(k_rows_apply<double, 8>, static_cast<double*>(Out));
+  else if (vt == EIG_F64) go(k_rows_apply<double, 16>, static_cast<double*>(Out));
   else return EIG_EINVAL;
   EIG_LAUNCH_CHECK("k_rows_apply");
   return EIG_OK;

@@ -102,11 +102,11 @@ __device__ __forceinline__ int tile_index(const uint32_t* slot, const int32_t* t
 
 // CTA per row block, warp per row (32 rows each), the row block's upper tiles (256 rows x 64 columns) in
 // groups of kCountTiles.  Per tile: seg[t * 256 + row] (unless seg is null), the offset in its row of the
-// row's first entry in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper entries of each
-// column (integer atomics in shared memory: order independent); the largest total of a tile; and, in the
-// bitmap of the full matrix, the transposed tiles (64 rows of this row block as a column block of the
-// row block that holds the tile's columns).  A group takes up each row where the group before it left
-// it, so that a row is read once however many groups there are.
+// row's first entry in the tile (preset to "none" where there is none); cnt[t * 64 + j], the strictly-upper
+// entries of each column (integer atomics in shared memory: order independent); the largest total of a
+// tile; and, in the bitmap of the full matrix, the transposed tiles (64 rows of this row block as a column
+// block of the row block that holds the tile's columns).  A group takes up each row where the group before
+// it left it, so that a row is read once however many groups there are.
 constexpr int kCountTiles = 32;
 __global__ void __launch_bounds__(kMR) k_mir_colcounts(int64_t n, const int64_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ col,
@@ -587,8 +587,8 @@ struct StreamRow {
 // Places the 32 rows of a stream of nblk blocks from blk0 on, LR lanes a row (32, or 8: four rows at a
 // time, which then have at most 8 * LR entries).  rv, rc: the warp's rows in shared memory, places: 8 each.
 template <typename V, int LR>
-__device__ __forceinline__ void scatter_rows(const ScatterArgs<V>& a, const StreamRow& mine, int64_t blk0, int nblk, V* rv0,
-                                             uint16_t* rc0, ClassPlace* places) {
+__device__ __forceinline__ void scatter_rows(const ScatterArgs<V>& a, const StreamRow& mine, int64_t blk0, int nblk,
+                                             V* rv0, uint16_t* rc0, ClassPlace* places) {
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int E = BlkPiece<V>::kEpp;
   const int lane = threadIdx.x & 31, sub = lane % LR, first = lane - sub, cls = lane & 7;
@@ -674,7 +674,8 @@ __device__ __forceinline__ void scatter_rows(const ScatterArgs<V>& a, const Stre
       *reinterpret_cast<uint4*>(a.bcol + at + l * kBS) = *reinterpret_cast<const uint4*>(rc + b * kBS);
 #pragma unroll
       for (int u = 0; u < kBS; u += E)
-        *reinterpret_cast<uint4*>(a.bval + at + blk_value_at<V>(l, u)) = *reinterpret_cast<const uint4*>(rv + b * kBS + u);
+        *reinterpret_cast<uint4*>(a.bval + at + blk_value_at<V>(l, u)) =
+            *reinterpret_cast<const uint4*>(rv + b * kBS + u);
     }
     __syncwarp();
   }
@@ -693,15 +694,13 @@ __host__ __device__ constexpr int scatter_cap(int steps) {
   return steps > few ? steps : few;
 }
 template <typename V, bool FEW>
-__global__ void __launch_bounds__(kMR, 4) k_rs_scatter(const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol,
-                                                    const V* __restrict__ lval, const int64_t* __restrict__ rowptr,
-                                                    const int32_t* __restrict__ col, const V* __restrict__ val, int64_t n,
-                                                    const int32_t* __restrict__ rbp, const int32_t* __restrict__ pan_rb,
-                                                    const int32_t* __restrict__ pt0, const int32_t* __restrict__ pnt,
-                                                    const int32_t* __restrict__ tcol, const uint16_t* __restrict__ cnt,
-                                                    const uint16_t* __restrict__ cntl, const uint8_t* __restrict__ perm,
-                                                    const int64_t* __restrict__ sboff, int pr, int cap,
-                                                    uint16_t* __restrict__ bcol, V* __restrict__ bval) {
+__global__ void __launch_bounds__(kMR, 4)
+k_rs_scatter(const int64_t* __restrict__ lptr, const int32_t* __restrict__ lcol, const V* __restrict__ lval,
+             const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, const V* __restrict__ val, int64_t n,
+             const int32_t* __restrict__ rbp, const int32_t* __restrict__ pan_rb, const int32_t* __restrict__ pt0,
+             const int32_t* __restrict__ pnt, const int32_t* __restrict__ tcol, const uint16_t* __restrict__ cnt,
+             const uint16_t* __restrict__ cntl, const uint8_t* __restrict__ perm, const int64_t* __restrict__ sboff,
+             int pr, int cap, uint16_t* __restrict__ bcol, V* __restrict__ bval) {
   static_assert(kBS == 8 && (kBS * sizeof(V)) % 16 == 0 && kW == 8, "a lane's block is whole 16-byte pieces");
   extern __shared__ __align__(16) unsigned char sm_rows[];
   __shared__ int32_t s_tc[32];
@@ -928,7 +927,8 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
   //    block without tiles still gets one empty panel so that its rows are written)
   std::vector<int64_t> h_tptr;
   std::vector<int32_t> h_tcol;
-  EIG_TRY(tile_lists_from_bitmap(nRB, wpr, bitmap, tmp.rb_cnt.as<int64_t>(), st, tmp.rb_ptr, P->m_tcol, h_tptr, h_tcol));
+  EIG_TRY(tile_lists_from_bitmap(nRB, wpr, bitmap, tmp.rb_cnt.as<int64_t>(), st, tmp.rb_ptr, P->m_tcol, h_tptr,
+                                 h_tcol));
   tiles.mem.release();   // the lists' copies waited for the kernels above; the streams may need the room
   std::vector<int32_t> rbp(nRB + 1, 0), pt0, pnt;
   for (int64_t I = 0; I < nRB; ++I) {
@@ -949,8 +949,9 @@ eig_status rowstream_fill(SpmmPlan* P, TileTemps& tiles, PlanTemps& tmp, cudaStr
   P->m_pr = std::max(1, *std::max_element(pnt.begin(), pnt.end())) * kMC;
   P->m_groups = row_groups(nRB);
   at = 0;
-  EIG_TRY(P->m_own.reserve(DevBuf::part(nRB * 16) + DevBuf::part((nRB + 1) * 4) + 2 * DevBuf::part(npan * 4) + DevBuf::part(npan * kMR) +
-                           DevBuf::part(npan * kW * 4) + DevBuf::part((npan * kW + 1) * 8)));
+  EIG_TRY(P->m_own.reserve(DevBuf::part(nRB * 16) + DevBuf::part((nRB + 1) * 4) + 2 * DevBuf::part(npan * 4) +
+                           DevBuf::part(npan * kMR) + DevBuf::part(npan * kW * 4) +
+                           DevBuf::part((npan * kW + 1) * 8)));
   P->m_order.borrow(P->m_own, nRB * 16, &at);
   P->m_rbp.borrow(P->m_own, (nRB + 1) * 4, &at);
   P->m_pt0.borrow(P->m_own, npan * 4, &at);
