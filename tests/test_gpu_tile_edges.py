@@ -407,3 +407,28 @@ def test_plan_memory_of_half_layout():
     want[:-64] += v[64:]
     want[64:] += v[:-64]
     assert np.array_equal(y.cpu().numpy()[:, 0], want)
+
+
+# the lower triangle of full and nearly full tiles (an offset per tile and row; rows of more than the 24
+# entries that the lanes keep in registers), either side of the mean fill from which it is built that way,
+# with a ragged last row block and column block; small integers, exact in any order
+@pytest.mark.parametrize("density", [0.15, 0.25, 0.6, 1.0])
+@pytest.mark.parametrize("val,dt", [("f32", torch.float32), ("bf16", torch.float32), ("f64", torch.float64)])
+@pytest.mark.parametrize("n", [300, 9 * 256 + 37])
+def test_plan_dense_tiles_exact(density, val, dt, n):
+    import oracle as O
+    from gen.synth import CSRUpper, round_to_storage
+    from paper_2305_15552_gb300 import binding as B
+    rng = np.random.default_rng(n)
+    D = np.triu(rng.random((n, n)) < density)
+    D[np.arange(0, n, 5), np.arange(0, n, 5)] = False       # rows without a diagonal
+    r, c = np.nonzero(D)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(r, minlength=n), out=rowptr[1:])
+    v = round_to_storage(rng.integers(1, 4, r.size).astype(np.float64), val)
+    H = CSRUpper(n=n, rowptr=rowptr, col=c.astype(np.int32), val=v, storage=val)
+    X = torch.tensor(rng.integers(-3, 4, (n, 8)), dtype=dt, device="cuda")
+    P = B.SpmmPlan(H, layout="mirrored")
+    Y = P.spmm(X).double().cpu().numpy()
+    P.close()
+    assert np.array_equal(Y, O.sym_upper_matmul(H, X.double().cpu().numpy()))
